@@ -263,6 +263,11 @@ def layout_shape(layout: int, w: int, h: int, n: int) -> tuple:
     return (n, n, h, w, 4)
 
 
+def _padded(layout: int, w: int, h: int) -> bool:
+    """Whether a buffer of the layout holds texels of no bucket (quads with an odd side)."""
+    return layout == RT_LAYOUT_QUADS and (w % 2 == 1 or h % 2 == 1)
+
+
 def layout_numel(layout: int, w: int, h: int, n: int) -> int:
     return int(np.prod(layout_shape(layout, w, h, n)))
 
@@ -291,7 +296,8 @@ def rt_read_texture(ctx: Context, obj_id: int, dst_layout: int = RT_LAYOUT_ATLAS
     shape = layout_shape(dst_layout, w, h, n)
     if fmt == RT_BIT1:  # one byte (0 or 1) per texel, no channels
         shape = shape[:-1]
-    codes = torch.zeros(shape, dtype=CODE_DTYPE[fmt], device=dev)  # the padding of quads stays zero
+    make = torch.zeros if _padded(dst_layout, w, h) else torch.empty  # the padding of quads stays zero
+    codes = make(shape, dtype=CODE_DTYPE[fmt], device=dev)
     scales = torch.empty((h, w), dtype=torch.float32, device=dev) if fmt == RT_E4M3_BUCKET_SCALE else None
     _lib.call("rt_read_texture", ctx.handle, int(obj_id), int(dst_layout), _ptr(codes), _ptr(scales),
               _stream(stream, dev))
@@ -665,8 +671,9 @@ def rt_convert_layout(src: torch.Tensor, src_layout: int, dst_layout: int, w: in
     _check(src, "src", torch.float32)
     if src.numel() != layout_numel(src_layout, w, h, n):
         raise ValueError("src must be shaped by layout_shape(src_layout, w, h, n)")
-    if dst is None:  # zeros: the padding of a quads buffer is not written
-        dst = torch.zeros(layout_shape(dst_layout, w, h, n), dtype=torch.float32, device=src.device)
+    if dst is None:  # zeros where there is padding: it is not written
+        make = torch.zeros if _padded(dst_layout, w, h) else torch.empty
+        dst = make(layout_shape(dst_layout, w, h, n), dtype=torch.float32, device=src.device)
     _check(dst, "dst", torch.float32)
     if dst.numel() != layout_numel(dst_layout, w, h, n):
         raise ValueError("dst must be shaped by layout_shape(dst_layout, w, h, n)")

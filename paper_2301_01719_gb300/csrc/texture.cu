@@ -12,22 +12,150 @@ constexpr int kThreads = 256;
 
 static inline unsigned blocks_for(int64_t items) { return (unsigned)((items + kThreads - 1) / kThreads); }
 
-// FP32 source (any layout) -> FP32 / FP16 / BF16 storage in dst_layout (PLANES
-// or QUADS), one thread per texel (the padding of a QUADS buffer is not written).
-__global__ void encode_elementwise(const float4* __restrict__ src, int src_layout, void* __restrict__ dst,
-                                   int dst_layout, int W, int H, int n, int fmt, int64_t total) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// ---------------------------------------------------------------------------
+// Copies between layouts: encoding a source, reading codes back, converting an
+// FP32 buffer.  S is the source's texel type, D the destination's, and Op
+// converts one texel.  Both kernels leave the padding of a QUADS destination
+// unwritten.
+// ---------------------------------------------------------------------------
+struct CopyTexel {
+    template <typename T>
+    __device__ __forceinline__ T operator()(T v) const {
+        return v;
+    }
+};
+struct EncodeF16 {
+    __device__ __forceinline__ uint2 operator()(float4 v) const { return pack_f16(v); }
+};
+struct EncodeBF16 {
+    __device__ __forceinline__ uint2 operator()(float4 v) const { return pack_bf16(v); }
+};
+
+// A block moves tiles of 32 x 2 buckets at one in-bucket row t and up to 16
+// in-bucket columns s through shared memory, reading in the order of the source
+// and writing in the order of the destination: a tile is runs of 32 buckets
+// (PLANES), of 16 quads (QUADS) or of 32 sc texels (ATLAS) on either side, so
+// both sides move whole cache lines.  Bound: HBM.  One thread per texel in
+// plane order instead stores every texel of an ATLAS destination n texels from
+// the next thread's (8 of each 32-byte sector).  1024^2 x 16^2 codes from QUADS
+// to ATLAS: FP16 4.76 -> 0.79 ms (5.4 TB/s read + written), E4M3 0.72 ms (the
+// index arithmetic starts to show), FP32 1.21 ms (7.1 TB/s).
+constexpr int kTileI = 32, kTileS = 16;
+constexpr int kTileRow = 40;               // shared-memory pitch of the second bucket row
+constexpr int kTilePitch = 2 * kTileRow - 7;  // and of the next s: 73, odd
+
+struct RelayoutShape {
+    int W, H, n, sc;             // sc: in-bucket columns per tile, the last chunk may hold fewer
+    int ti, tj, chunks;          // tiles along i and j, chunks of s
+    FastDiv div_sc;
+    int step_b, step_s;          // kThreads = step_b sc + step_s
+};
+
+static RelayoutShape relayout_shape(int W, int H, int n) {
+    RelayoutShape r;
+    r.W = W;
+    r.H = H;
+    r.n = n;
+    r.chunks = (n + kTileS - 1) / kTileS;
+    r.sc = (n + r.chunks - 1) / r.chunks;
+    r.ti = (W + kTileI - 1) / kTileI;
+    r.tj = (H + 1) / 2;
+    r.div_sc = make_fastdiv((uint32_t)r.sc);
+    r.step_b = kThreads / r.sc;
+    r.step_s = kThreads % r.sc;
+    return r;
+}
+
+// Calls f(offset of the texel in the buffer, its place in the tile) for this
+// thread's texels of the tile, in the buffer's order: texels threadIdx.x,
+// threadIdx.x + kThreads, ... of 64 sc, stepped without divisions.
+template <typename F>
+__device__ __forceinline__ void for_tile_texels(int layout, const RelayoutShape& r, int i0, int j0, int t, int s0,
+                                                F f) {
+    constexpr int kSteps = 2 * kTileI * kTileS / kThreads;
+    const int sc = min(r.sc, r.n - s0);
+    if (layout == RT_LAYOUT_ATLAS) {
+        const int64_t row = (int64_t)r.W * r.n;
+        const int64_t base = ((int64_t)j0 * r.n + t) * row + (int64_t)i0 * r.n + s0;
+        const int64_t next = row * r.n;  // from bucket row j0 to j0 + 1
+        int b = (int)r.div_sc.div(threadIdx.x), s = (int)threadIdx.x - b * r.sc;
+#pragma unroll
+        for (int k = 0; k < kSteps; ++k) {
+            const int ii = b & (kTileI - 1), jj = b / kTileI;
+            if (jj < 2 && s < sc && i0 + ii < r.W && j0 + jj < r.H)
+                f(base + (jj ? next : 0) + ii * r.n + s, s * kTilePitch + jj * kTileRow + ii);
+            b += r.step_b;
+            s += r.step_s;
+            if (s >= r.sc) {
+                s -= r.sc;
+                ++b;
+            }
+        }
+    } else {
+        // kThreads is a multiple of 64: a thread keeps its bucket and takes every fourth s
+        const bool quads = layout == RT_LAYOUT_QUADS;
+        const int64_t plane = plane_buckets(layout, r.W, r.H);
+        const int q = threadIdx.x & (2 * kTileI - 1), s1 = threadIdx.x / (2 * kTileI);
+        const int jj = quads ? (q >> 1) & 1 : q / kTileI;
+        const int ii = quads ? ((q >> 2) << 1) + (q & 1) : q & (kTileI - 1);
+        if (i0 + ii >= r.W || j0 + jj >= r.H) return;
+        int64_t o = ((int64_t)t * r.n + s0 + s1) * plane + slot_in(layout, r.W, i0 + ii, j0 + jj);
+        int p = s1 * kTilePitch + jj * kTileRow + ii;
+#pragma unroll
+        for (int k = 0; k < kSteps; ++k) {
+            if (s1 + k * (kThreads / (2 * kTileI)) < sc) f(o, p);
+            o += (kThreads / (2 * kTileI)) * plane;
+            p += (kThreads / (2 * kTileI)) * kTilePitch;
+        }
+    }
+}
+
+template <typename S, typename D, typename Op>
+__global__ void __launch_bounds__(kThreads, 6) relayout_tiles(const S* __restrict__ src, int src_layout,
+                                                           D* __restrict__ dst, int dst_layout, RelayoutShape r) {
+    __shared__ D tile[kTileS * kTilePitch];
+    const Op op;
+    const int tj = (int)(blockIdx.x / (unsigned)r.ti), t = (int)(blockIdx.y / (unsigned)r.chunks);
+    const int i0 = (int)(blockIdx.x - (unsigned)tj * r.ti) * kTileI, j0 = 2 * tj;
+    const int s0 = (int)(blockIdx.y - (unsigned)t * r.chunks) * r.sc;
+    for_tile_texels(src_layout, r, i0, j0, t, s0, [&](int64_t o, int p) { tile[p] = op(src[o]); });
+    __syncthreads();
+    for_tile_texels(dst_layout, r, i0, j0, t, s0, [&](int64_t o, int p) { dst[o] = tile[p]; });
+}
+
+// One thread per texel in plane order, for narrow bucket matrices, which leave
+// most of a tile empty.
+template <typename S, typename D, typename Op>
+__global__ void relayout_texels(const S* __restrict__ src, int src_layout, D* __restrict__ dst, int dst_layout, int W,
+                                int H, int n, int64_t total) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= total) return;
     int i, j, s, t;
     planes_coords(idx, W, H, n, i, j, s, t);
-    const float4 v = src[index_in(src_layout, W, H, n, i, j, s, t)];
-    const int64_t o = index_in(dst_layout, W, H, n, i, j, s, t);
-    if (fmt == RT_F32)
-        reinterpret_cast<float4*>(dst)[o] = v;
-    else if (fmt == RT_F16)
-        reinterpret_cast<uint2*>(dst)[o] = pack_f16(v);
-    else
-        reinterpret_cast<uint2*>(dst)[o] = pack_bf16(v);
+    dst[index_in(dst_layout, W, H, n, i, j, s, t)] = Op()(src[index_in(src_layout, W, H, n, i, j, s, t)]);
+}
+
+// FP32, 2^17 buckets x 16^2, tiles against one thread per texel: 16 wide 311 /
+// 476 us (QUADS to ATLAS) but 258 / 195 us (PLANES to QUADS), 24 wide 164 / 472
+// and 159 / 195, 8 wide 545 / 492 and 473 / 195.
+constexpr int kTileMinWidth = 24;
+
+template <typename S, typename D, typename Op = CopyTexel>
+static cudaError_t launch_relayout(const void* src, int src_layout, void* dst, int dst_layout, int W, int H, int n,
+                                   cudaStream_t stream) {
+    const S* s = static_cast<const S*>(src);
+    D* d = static_cast<D*>(dst);
+    if (W >= kTileMinWidth) {
+        const RelayoutShape r = relayout_shape(W, H, n);
+        // w h <= 2^30 (or a K x 1 palette, K <= 2^30) and n <= 64: at most 2^25 x 256 blocks
+        const dim3 grid((unsigned)r.ti * (unsigned)r.tj, (unsigned)(n * r.chunks));
+        relayout_tiles<S, D, Op><<<grid, kThreads, 0, stream>>>(s, src_layout, d, dst_layout, r);
+    } else {
+        const int64_t total = (int64_t)W * H * n * n;
+        relayout_texels<S, D, Op><<<blocks_for(total), kThreads, 0, stream>>>(s, src_layout, d, dst_layout, W, H, n,
+                                                                              total);
+    }
+    return cudaGetLastError();
 }
 
 // FP32 source -> E4M3 + per-bucket scale (stored at the bucket's slot of
@@ -74,25 +202,14 @@ cudaError_t launch_encode(const float* src, int src_layout, void* dst, float* sc
         encode_e4m3_buckets<<<blocks_for(buckets), kThreads, 0, stream>>>(
             reinterpret_cast<const float4*>(src), src_layout, reinterpret_cast<unsigned*>(dst), scale, dst_layout, W,
             H, n);
+    } else if (fmt == RT_F32) {
+        return launch_relayout<float4, float4>(src, src_layout, dst, dst_layout, W, H, n, stream);
+    } else if (fmt == RT_F16) {
+        return launch_relayout<float4, uint2, EncodeF16>(src, src_layout, dst, dst_layout, W, H, n, stream);
     } else {
-        int64_t total = (int64_t)W * H * n * n;
-        encode_elementwise<<<blocks_for(total), kThreads, 0, stream>>>(reinterpret_cast<const float4*>(src),
-                                                                       src_layout, dst, dst_layout, W, H, n, fmt,
-                                                                       total);
+        return launch_relayout<float4, uint2, EncodeBF16>(src, src_layout, dst, dst_layout, W, H, n, stream);
     }
     return cudaGetLastError();
-}
-
-// Stored codes (src_layout: PLANES or QUADS) -> codes in dst_layout; T is the
-// per-texel code type; one thread per texel (padding is not written).
-template <typename T>
-__global__ void read_codes(const T* __restrict__ src, int src_layout, T* __restrict__ dst, int W, int H, int n,
-                           int dst_layout, int64_t total) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    int i, j, s, t;
-    planes_coords(idx, W, H, n, i, j, s, t);
-    dst[index_in(dst_layout, W, H, n, i, j, s, t)] = src[index_in(src_layout, W, H, n, i, j, s, t)];
 }
 
 // Per-bucket scales stored at their slots of src_layout -> row-major h x w.
@@ -114,22 +231,24 @@ __global__ void read_bits(const unsigned* __restrict__ src, uint8_t* __restrict_
     dst[o] = (uint8_t)((src[idx >> 5] >> (unsigned)(idx & 31)) & 1u);
 }
 
+// Stored codes (src_layout: PLANES or QUADS) -> codes in dst_layout.
 cudaError_t launch_read(const void* src, int src_layout, const float* scale, int fmt, int W, int H, int n,
                         int dst_layout, void* dst, float* scale_dst, cudaStream_t stream) {
-    int64_t total = (int64_t)W * H * n * n;
-    unsigned g = blocks_for(total);
-    if (fmt == RT_BIT1)  // bit textures are always PLANES
-        read_bits<<<g, kThreads, 0, stream>>>(reinterpret_cast<const unsigned*>(src), reinterpret_cast<uint8_t*>(dst),
-                                              W, H, n, dst_layout, total);
-    else if (fmt == RT_F32)
-        read_codes<float4><<<g, kThreads, 0, stream>>>(reinterpret_cast<const float4*>(src), src_layout,
-                                                       reinterpret_cast<float4*>(dst), W, H, n, dst_layout, total);
-    else if (fmt == RT_E4M3_BUCKET_SCALE)
-        read_codes<unsigned><<<g, kThreads, 0, stream>>>(reinterpret_cast<const unsigned*>(src), src_layout,
-                                                         reinterpret_cast<unsigned*>(dst), W, H, n, dst_layout, total);
-    else
-        read_codes<uint2><<<g, kThreads, 0, stream>>>(reinterpret_cast<const uint2*>(src), src_layout,
-                                                      reinterpret_cast<uint2*>(dst), W, H, n, dst_layout, total);
+    cudaError_t e;
+    if (fmt == RT_BIT1) {  // bit textures are always PLANES
+        const int64_t total = (int64_t)W * H * n * n;
+        read_bits<<<blocks_for(total), kThreads, 0, stream>>>(reinterpret_cast<const unsigned*>(src),
+                                                              reinterpret_cast<uint8_t*>(dst), W, H, n, dst_layout,
+                                                              total);
+        e = cudaGetLastError();
+    } else if (fmt == RT_F32) {
+        e = launch_relayout<float4, float4>(src, src_layout, dst, dst_layout, W, H, n, stream);
+    } else if (fmt == RT_E4M3_BUCKET_SCALE) {
+        e = launch_relayout<unsigned, unsigned>(src, src_layout, dst, dst_layout, W, H, n, stream);
+    } else {
+        e = launch_relayout<uint2, uint2>(src, src_layout, dst, dst_layout, W, H, n, stream);
+    }
+    if (e != cudaSuccess) return e;
     if (scale && scale_dst)
         read_scales<<<blocks_for((int64_t)W * H), kThreads, 0, stream>>>(scale, src_layout, scale_dst, W, H);
     return cudaGetLastError();
@@ -181,15 +300,6 @@ cudaError_t launch_fill_lobes(const float* params, void* dst, float* scale, int 
     return cudaGetLastError();
 }
 
-__global__ void convert_kernel(const float4* __restrict__ src, int src_layout, float4* __restrict__ dst,
-                               int dst_layout, int W, int H, int n, int64_t total) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    int i, j, s, t;
-    planes_coords(idx, W, H, n, i, j, s, t);
-    dst[index_in(dst_layout, W, H, n, i, j, s, t)] = src[index_in(src_layout, W, H, n, i, j, s, t)];
-}
-
 __global__ void check_index_kernel(const uint32_t* __restrict__ index, int64_t count, uint32_t K, unsigned* bad) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < count && index[k] >= K) atomicOr(bad, 1u);
@@ -203,11 +313,7 @@ cudaError_t launch_check_index(const uint32_t* index, int64_t count, uint32_t K,
 
 cudaError_t launch_convert(const float* src, int src_layout, float* dst, int dst_layout, int W, int H, int n,
                            cudaStream_t stream) {
-    int64_t total = (int64_t)W * H * n * n;
-    convert_kernel<<<blocks_for(total), kThreads, 0, stream>>>(reinterpret_cast<const float4*>(src), src_layout,
-                                                               reinterpret_cast<float4*>(dst), dst_layout, W, H, n,
-                                                               total);
-    return cudaGetLastError();
+    return launch_relayout<float4, float4>(src, src_layout, dst, dst_layout, W, H, n, stream);
 }
 
 // Footprint: one bit per texel of every object (PLANES numbering), set for

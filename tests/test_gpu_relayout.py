@@ -1,0 +1,70 @@
+"""Copies between texture layouts at the edges of their tiles (32 x 2 buckets, up to 16 in-bucket
+columns): every texel must land at its layout's index, bit for bit, and the padding of a quads
+destination must stay as it was.  The reference is numpy's permutation of the atlas."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2301_01719_gb300 import api
+from parity_util import atlas_to_quads
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(1, 1, 1), (7, 3, 5), (8, 2, 16), (31, 1, 17), (32, 4, 16), (33, 5, 33), (64, 3, 64), (130, 2, 3), (9, 70, 15)]
+LAYOUTS = [api.RT_LAYOUT_ATLAS, api.RT_LAYOUT_PLANES, api.RT_LAYOUT_QUADS]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+def _in_layout(atlas, layout, w, h, n, pad=0):
+    """The (h n, w n, ...) atlas as an array of the layout's shape."""
+    tail = atlas.shape[2:]
+    planes = atlas.reshape(h, n, w, n, *tail).swapaxes(1, 2).transpose(2, 3, 0, 1, *range(4, 4 + len(tail)))
+    if layout == api.RT_LAYOUT_ATLAS:
+        return atlas
+    if layout == api.RT_LAYOUT_PLANES:
+        return np.ascontiguousarray(planes)
+    full = np.full((n, n, h + h % 2, w + w % 2, *tail), pad, dtype=atlas.dtype)
+    full[:, :, :h, :w] = planes
+    full = full.reshape(n, n, (h + 1) // 2, 2, (w + 1) // 2, 2, *tail)
+    return np.ascontiguousarray(full.swapaxes(3, 4))
+
+
+@pytest.mark.parametrize("w,h,n", SIZES)
+def test_convert_layout_moves_every_texel(ctx, w, h, n):
+    atlas = np.random.default_rng(w * 1000 + h * 10 + n).standard_normal((h * n, w * n, 4)).astype(np.float32)
+    np.testing.assert_array_equal(_in_layout(atlas, api.RT_LAYOUT_QUADS, w, h, n), atlas_to_quads(atlas, w, h, n))
+    for src in LAYOUTS:
+        a = torch.from_numpy(_in_layout(atlas, src, w, h, n, pad=7.0)).cuda()
+        for dst in LAYOUTS:
+            to = torch.full(api.layout_shape(dst, w, h, n), -3.0, device="cuda")
+            got = api.rt_convert_layout(a, src, dst, w, h, n, to)
+            np.testing.assert_array_equal(got.cpu().numpy(), _in_layout(atlas, dst, w, h, n, pad=-3.0))
+
+
+@pytest.mark.parametrize("w,h,n", SIZES)
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16", "e4m3"])
+def test_stored_codes_read_back_in_every_layout(ctx, w, h, n, storage):
+    atlas = np.random.default_rng(w + h + n).uniform(-2.0, 2.0, (h * n, w * n, 4)).astype(np.float32)
+    want = None
+    for src in LAYOUTS:
+        t = torch.from_numpy(_in_layout(atlas, src, w, h, n)).cuda()
+        oid = api.rt_create_texture(ctx, w, h, n, api.FORMAT_NAMES[storage], src, t)
+        codes = api.rt_read_texture(ctx, oid, api.RT_LAYOUT_ATLAS)[0].cpu().numpy()
+        if storage in ("f32", "f16", "bf16"):
+            kind = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}[storage]
+            enc = torch.from_numpy(atlas).to(kind)
+            want = enc.numpy() if storage == "f32" else enc.view(torch.int16).numpy()
+        want = codes if want is None else want  # E4M3: the same codes whatever the source's layout
+        np.testing.assert_array_equal(codes, want)
+        for dst in LAYOUTS[1:]:
+            got = api.rt_read_texture(ctx, oid, dst)[0].cpu().numpy()
+            np.testing.assert_array_equal(got, _in_layout(want, dst, w, h, n))
+        api.rt_destroy_texture(ctx, oid)
