@@ -6,6 +6,8 @@
 // one per tap of non-zero weight.  UV and direction gradients follow the chain
 // rule through the nested lerps, the Note's clamp (zero derivative where a
 // coordinate is clamped), Eq. 3 and Eq. 1b.
+#include <cmath>
+
 #include "launch.h"
 #include "rt_backward.cuh"
 #include "rt_internal.h"
@@ -15,7 +17,7 @@ namespace rt {
 // The single-format tiled kernels are held to 80 registers (6 blocks, 24 warps
 // per SM): measured 3 % faster than 95 registers at 5 blocks.
 template <int FILTER, bool TILED, bool DET, int SPEC>
-__global__ void __launch_bounds__(kBackThreads, (TILED && !DET && SPEC >= 0) ? 6 : 1) backward_kernel(
+__global__ void __launch_bounds__(kBackThreads, DET ? 4 : (TILED && SPEC >= 0) ? 6 : 1) backward_kernel(
     const TexDesc* __restrict__ table, int n_obj, const float* __restrict__ uv, const float* __restrict__ dir,
     const int32_t* __restrict__ obj, int64_t F, Tiling tiling, const float* __restrict__ dL_dout,
     const __grid_constant__ GradTable grads, bool any_grad, float* __restrict__ dL_duv, float* __restrict__ dL_ddir,
@@ -27,10 +29,19 @@ __global__ void __launch_bounds__(kBackThreads, (TILED && !DET && SPEC >= 0) ? 6
         float2 guv = make_float2(0.f, 0.f);
         float3 gdir = make_float3(0.f, 0.f, 0.f);
         TexDesc d;
-        if (fragment_valid(table, n_obj, q.o, q.u, q.v, q.x, q.y, q.z, status, d)) {
-            Lookup<FILTER> L = locate<FILTER, (SPEC < 0)>(d, q.u, q.v, q.x, q.y, q.z);
-            void* grad = any_grad ? grads.p[q.o] : nullptr;
-            CoordGrad cg = backward_spec<FILTER, DET, SPEC>(d, L, go, grad, coord_grads);
+        Lookup<FILTER> L;
+        void* grad = nullptr;
+        const bool valid = fragment_valid(table, n_obj, q.o, q.u, q.v, q.x, q.y, q.z, status, d);
+        if (valid) {
+            L = locate<FILTER, (SPEC < 0)>(d, q.u, q.v, q.x, q.y, q.z);
+            if (any_grad) grad = grads.p[q.o];
+        }
+        if (DET) {
+            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
+            grad = nullptr;
+        }
+        if (valid && (!DET || coord_grads)) {
+            CoordGrad cg = backward_spec<FILTER, SPEC>(d, L, go, grad, coord_grads);
             coord_grads_of<FILTER>(d, L, q, cg, dL_ddir != nullptr, guv, gdir);
         }
         if (f < 0) return;
@@ -119,10 +130,20 @@ __global__ void __launch_bounds__(kBackThreads) world_backward_kernel(
         float3 gh = make_float3(0.f, 0.f, 0.f);
         TexDesc d;
         const float3 I = make_float3(q.x, q.y, q.z), N = make_float3(q.nx, q.ny, q.nz);
-        if (fragment_valid(table, n_obj, q.o, q.u, q.v, I.x, I.y, I.z, status, d) && normal_valid(N, status)) {
-            const Lookup<FILTER> L = locate_world<FILTER>(d, q.u, q.v, I, N);
-            void* grad = any_grad ? grads.p[q.o] : nullptr;
-            const CoordGrad cg = backward_any<FILTER, DET>(d, L, go, grad, coord_grads);
+        Lookup<FILTER> L;
+        void* grad = nullptr;
+        const bool valid = fragment_valid(table, n_obj, q.o, q.u, q.v, I.x, I.y, I.z, status, d) &&
+                           normal_valid(N, status);
+        if (valid) {
+            L = locate_world<FILTER>(d, q.u, q.v, I, N);
+            if (any_grad) grad = grads.p[q.o];
+        }
+        if (DET) {
+            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
+            grad = nullptr;
+        }
+        if (valid && (!DET || coord_grads)) {
+            const CoordGrad cg = backward_any<FILTER>(d, L, go, grad, coord_grads);
             if (FILTER == RT_QUADRILINEAR) guv = uv_grad(d, q.u, q.v, cg.gu, cg.gv);
             if (FILTER != RT_NEAREST && (dL_ddir || dL_dnrm)) {
                 const float gBx = (L.B.x > -d.hi && L.B.x < d.hi) ? cg.gs * d.half_n : 0.f;
@@ -200,23 +221,87 @@ cudaError_t launch_world_backward(const TexDesc* table, int n_obj, const float* 
 #undef RT_WBWD_D
 }
 
-// Fixed-point sums (deterministic mode) -> FP32 gradients, times `scale` (the
-// product taken in FP64, rounded once), added to or overwriting dst.
-__global__ void fixed_to_float_kernel(const long long* __restrict__ acc, float* __restrict__ dst, int64_t count,
-                                      double scale, bool accumulate) {
-    const double f = scale * (1.0 / 4294967296.0);
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (int64_t)gridDim.x * blockDim.x) {
-        float v = (float)((double)acc[k] * f);
-        dst[k] = accumulate ? dst[k] + v : v;
+// Fixed-point sums (deterministic mode) -> FP32 gradients: the sum times
+// f = scale 2^-32, the product rounded to FP64 and then to FP32, added to or
+// overwriting dst.  The FP64 pipe takes a few operations per cycle and SM, and
+// converting to double, multiplying and converting back would bound the pass at
+// three times its memory time.  So a magnitude below 2^52 becomes the mantissa
+// of 2^52 + |a|, one FMA takes (2^52 + |a|) |f| - 2^52 |f| = |a| |f| with the
+// one rounding a product has, and FP32 is rounded from its bits in integers.
+struct FixedScale {
+    double f, mag, minus;  // f, |f| and -2^52 |f|
+    uint32_t sign;         // f's sign, in bit 31
+};
+
+static FixedScale fixed_scale(double scale) {
+    FixedScale s;
+    s.f = scale * (1.0 / 4294967296.0);
+    s.mag = std::fabs(s.f);
+    s.minus = -4503599627370496.0 * s.mag;  // infinite for a huge scale: no product of it passes the test below
+    s.sign = std::signbit(s.f) ? 0x80000000u : 0u;
+    return s;
+}
+
+// A call, so that the compiler does not compute it beside the other form.
+__device__ __noinline__ float fixed_to_float_any(long long a, double f) { return (float)((double)a * f); }
+
+__device__ __forceinline__ float fixed_to_float(long long a, const FixedScale& s) {
+    const uint32_t sign = (a < 0 ? 0x80000000u : 0u) ^ s.sign;
+    const uint64_t m = a < 0 ? 0ull - (uint64_t)a : (uint64_t)a;
+    if (m == 0) return __uint_as_float(sign);
+    const double d = __fma_rn(__longlong_as_double((long long)(m | 0x4330000000000000ull)), s.mag, s.minus);
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t e = hi >> 20;  // d >= 0; an FP32 in its normal range for e in [897, 1150)
+    if (m < (1ull << 52) && e - 897u < 253u) {
+        const uint32_t y = __funnelshift_l(lo, hi, 3) - 0xC0000000u;  // the bits above the lowest 29, rebiased
+        const uint32_t up = ((lo & 0x1fffffffu) + 0x0fffffffu + (y & 1u)) >> 29;
+        return __uint_as_float(sign | (y + up));
+    }
+    return fixed_to_float_any(a, s.f);
+}
+
+// Two values per thread and load, so that a warp's loads (512 bytes) and stores
+// (256) are whole lines, four loads in flight (acc and dst 16-byte aligned);
+// an odd last value by itself.  Bound: HBM.  151 M values (1.8 GB): 0.83 ms with
+// one value per thread and three FP64 operations each, 0.25-0.27 ms here.
+constexpr int kFixedUnroll = 4;
+
+__global__ void __launch_bounds__(256) fixed_to_float_kernel(const long long* __restrict__ acc,
+                                                             float* __restrict__ dst, int64_t count, FixedScale f,
+                                                             bool accumulate) {
+    const longlong2* in = reinterpret_cast<const longlong2*>(acc);
+    float2* out = reinterpret_cast<float2*>(dst);
+    const int64_t pairs = count / 2, first = (int64_t)blockIdx.x * (blockDim.x * kFixedUnroll) + threadIdx.x;
+    longlong2 a[kFixedUnroll];
+#pragma unroll
+    for (int u = 0; u < kFixedUnroll; ++u) {
+        const int64_t k = first + u * 256;
+        a[u] = k < pairs ? __ldcs(in + k) : make_longlong2(0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < kFixedUnroll; ++u) {
+        const int64_t k = first + u * 256;
+        if (k >= pairs) break;
+        float2 v = make_float2(fixed_to_float(a[u].x, f), fixed_to_float(a[u].y, f));
+        if (accumulate) {
+            const float2 o = out[k];
+            v = make_float2(o.x + v.x, o.y + v.y);
+        }
+        out[k] = v;
+    }
+    if (first == 0 && (count & 1)) {
+        const float v = fixed_to_float(acc[count - 1], f);
+        dst[count - 1] = accumulate ? dst[count - 1] + v : v;
     }
 }
 
 cudaError_t launch_fixed_to_float(const long long* acc, float* dst, int64_t count, bool accumulate,
                                   cudaStream_t stream, double scale) {
     if (count <= 0) return cudaSuccess;
-    int64_t blocks = (count + 255) / 256;
-    fixed_to_float_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, stream>>>(acc, dst, count, scale,
-                                                                                          accumulate);
+    const int64_t blocks = (count / 2 + 256 * kFixedUnroll - 1) / (256 * kFixedUnroll);
+    if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+    fixed_to_float_kernel<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, stream>>>(acc, dst, count,
+                                                                                 fixed_scale(scale), accumulate);
     return cudaGetLastError();
 }
 

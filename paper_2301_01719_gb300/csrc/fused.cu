@@ -46,7 +46,7 @@ __device__ __forceinline__ P4 decode_kept(typename KeptCode<FMT>::type c, float 
 // registers and measured slower at every occupancy (7.0 ms at best against
 // 6.4 ms then).
 template <int FILTER, bool DET, int SPEC>
-__global__ void __launch_bounds__(kBackThreads, (!DET && SPEC >= 0) ? 4 : 1) fused_l2_kernel(
+__global__ void __launch_bounds__(kBackThreads, (DET || SPEC >= 0) ? 4 : 1) fused_l2_kernel(
     const TexDesc* __restrict__ table, int n_obj, const float* __restrict__ uv, const float* __restrict__ dir,
     const int32_t* __restrict__ obj, int64_t F, Tiling tiling, const float* __restrict__ target, float scale,
     float* __restrict__ out, double* __restrict__ sums, const __grid_constant__ GradTable grads, bool any_grad,
@@ -103,18 +103,22 @@ __global__ void __launch_bounds__(kBackThreads, (!DET && SPEC >= 0) ? 4 : 1) fus
         }
         float2 guv = make_float2(0.f, 0.f);
         float3 gdir = make_float3(0.f, 0.f, 0.f);
-        if (valid) {
-            const float4 g = make_float4(scale * (c.x - t.x), scale * (c.y - t.y), scale * (c.z - t.z),
-                                         scale * (c.w - t.w));
-            void* grad = any_grad ? grads.p[q.o] : nullptr;
+        const float4 g = make_float4(scale * (c.x - t.x), scale * (c.y - t.y), scale * (c.z - t.z),
+                                     scale * (c.w - t.w));
+        void* grad = valid && any_grad ? grads.p[q.o] : nullptr;
+        if (DET) {
+            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, g, grad, status);
+            grad = nullptr;
+        }
+        if (valid && (!DET || coord_grads)) {
             CoordGrad cg;
             if constexpr (kKeepTaps) {
-                reduce_quadrilinear_taps<false>(d, L, pl, o, g, grad);
+                reduce_quadrilinear_taps(d, L, pl, o, g, grad);
                 cg = CoordGrad{0.f, 0.f, 0.f, 0.f};
                 if (coord_grads)
                     cg = quad_coord_grads(L, g, [&](int b, int k) { return decode_kept<kKept>(code[b][k], sc[kE4 ? b : 0]); });
             } else {
-                cg = backward_spec<FILTER, DET, SPEC>(d, L, g, grad, coord_grads);
+                cg = backward_spec<FILTER, SPEC>(d, L, g, grad, coord_grads);
             }
             coord_grads_of<FILTER>(d, L, q, cg, dL_ddir != nullptr, guv, gdir);
         }
@@ -174,7 +178,7 @@ cudaError_t launch_fused_l2(const TexDesc* table, int n_obj, const float* uv, co
 #define RT_FUSED(DET, SPEC)                                                                                         \
     launch_fused_f<DET, SPEC>(table, n_obj, uv, dir, obj, F, filter, T, target, scale, out, sums, grads, any_grad,  \
                               dL_duv, dL_ddir, accumulate, status, stream)
-    if (deterministic) return RT_FUSED(true, -1);
+    if (deterministic) return spec == RT_F32 ? RT_FUSED(true, RT_F32) : RT_FUSED(true, -1);  // fitting: FP32
     switch (spec) {
         case RT_F16:
             return RT_FUSED(false, RT_F16);

@@ -24,11 +24,152 @@ struct CoordGrad {
 // which fragments arrive.
 constexpr float kFixedScale = 4294967296.0f;  // 2^32
 
-__device__ __forceinline__ void red_add_fixed4(unsigned long long* addr, float4 v) {
-    atomicAdd(addr + 0, (unsigned long long)__float2ll_rn(v.x * kFixedScale));
-    atomicAdd(addr + 1, (unsigned long long)__float2ll_rn(v.y * kFixedScale));
-    atomicAdd(addr + 2, (unsigned long long)__float2ll_rn(v.z * kFixedScale));
-    atomicAdd(addr + 3, (unsigned long long)__float2ll_rn(v.w * kFixedScale));
+// round(v 2^32) to nearest even, |v| < 2^31.
+__device__ __forceinline__ unsigned long long to_fixed_any(float v) {
+    return (unsigned long long)__float2ll_rn(v * kFixedScale);
+}
+
+// The same for |v| <= kFixedSmall.  Conversions to 64-bit integers run on the
+// FP64 pipe (a few per cycle and SM), so this takes two FP32 roundings instead:
+// q = v 2^10 to an integer by adding 1.5 2^23 (its low mantissa bits), the
+// remainder v - q 2^-10 (exact: at most 24 bits lie between 2^-11 and the last
+// bit of v), and that times 2^32 to an integer the same way; q 2^22 is even, so
+// ties fall as they do for the whole.
+constexpr float kFixedSmall = 4096.0f;
+
+__device__ __forceinline__ unsigned long long to_fixed_small(float v) {
+    constexpr float kMagic = 12582912.0f;  // 1.5 2^23
+    const float q = __fmaf_rn(v, 1024.0f, kMagic);
+    const float rem = __fmaf_rn(__fsub_rn(q, kMagic), -1.0f / 1024.0f, v);
+    const float t = __fmaf_rn(rem, kFixedScale, kMagic);
+    const int qi = __float_as_int(q) - __float_as_int(kMagic), ti = __float_as_int(t) - __float_as_int(kMagic);
+    return (unsigned long long)((long long)qi * (1 << 22) + ti);
+}
+
+// The taps of a lookup as two sums: tap (b, k) is texel bucket[b] + texel[k],
+// for every layout.
+template <int FILTER>
+struct TapTable {
+    static constexpr int kBuckets = FILTER == RT_QUADRILINEAR ? 4 : 1;  // (u0,v0) (u1,v0) (u0,v1) (u1,v1)
+    static constexpr int kTexels = FILTER == RT_NEAREST ? 1 : 4;        // (s0,t0) (s1,t0) (s0,t1) (s1,t1)
+    int64_t bucket[kBuckets];
+    int64_t texel[kTexels];
+};
+
+template <int FILTER, int LAYOUT>
+__device__ __forceinline__ void bucket_offsets(const TexDesc& d, const Lookup<FILTER>& L, TapTable<FILTER>& T) {
+    if constexpr (FILTER == RT_QUADRILINEAR) {
+        int o[4];
+        bucket_slots4<LAYOUT>(d, L.u.k0, L.u.k1, L.v.k0, L.v.k1, o);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) T.bucket[b] = o[b];
+    } else {
+        T.bucket[0] = bucket_slot<LAYOUT>(d, L.u.k0, L.v.k0);
+    }
+}
+
+template <int FILTER>
+__device__ __forceinline__ void tap_table(const TexDesc& d, const Lookup<FILTER>& L, TapTable<FILTER>& T) {
+    const bool atlas = d.layout == RT_LAYOUT_ATLAS;
+    const int64_t ps = atlas ? 1 : d.plane, pt = atlas ? (int64_t)d.W * d.n : d.plane * d.n;
+#pragma unroll
+    for (int k = 0; k < T.kTexels; ++k) T.texel[k] = ((k & 1) ? L.s.k1 : L.s.k0) * ps + ((k >> 1) ? L.t.k1 : L.t.k0) * pt;
+    if (atlas) {
+#pragma unroll
+        for (int b = 0; b < T.kBuckets; ++b)
+            T.bucket[b] = (((b >> 1) ? L.v.k1 : L.v.k0) * pt + ((b & 1) ? L.u.k1 : L.u.k0)) * d.n;
+    } else if (d.layout == RT_LAYOUT_QUADS) {
+        bucket_offsets<FILTER, RT_LAYOUT_QUADS>(d, L, T);
+    } else if (d.layout == kLayoutPalette) {
+        bucket_offsets<FILTER, kLayoutPalette>(d, L, T);
+    } else {
+        bucket_offsets<FILTER, RT_LAYOUT_PLANES>(d, L, T);
+    }
+}
+
+// Deterministic mode: the warp's texel gradients, all 32 lanes calling (`has`:
+// this lane's fragment has some).  A texel's four channels are four 64-bit
+// sums, one 32-byte sector.  Were each lane to add the four of its own
+// fragment, one atomic instruction would touch 32 sectors and L2, which takes a
+// sector per operation, would be asked four times for each.  So four lanes
+// share their four fragments: they take one fragment at a time, each its own
+// channel, and one instruction adds whole sectors.
+// On 12 views of 768^2 into 384^2 x 16^2 FP32 the fused step's kernel went from
+// 1.63 ms to 0.60 ms; adding the texels that horizontal neighbours share once (as
+// reduce_quadrilinear_taps does) took 0.94 ms, the partner's weights costing
+// more than the adds they save.
+template <int FILTER>
+__device__ __forceinline__ void reduce_fixed_warp(bool has, const TexDesc& d, const Lookup<FILTER>& L, float4 g,
+                                                  void* grad, unsigned* status) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (!__any_sync(kAll, has)) return;
+    const int lane = threadIdx.x & 31, c = lane & 3;
+    TapTable<FILTER> T;
+    if (has) tap_table<FILTER>(d, L, T);
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {
+        const int src = (lane & 28) | r;
+        const bool hr = __shfl_sync(kAll, (int)has, src) != 0;
+        char* base = reinterpret_cast<char*>(__shfl_sync(kAll, (unsigned long long)grad, src)) + 8 * c;
+        const float gx = __shfl_sync(kAll, g.x, src), gy = __shfl_sync(kAll, g.y, src);
+        const float gz = __shfl_sync(kAll, g.z, src), gw = __shfl_sync(kAll, g.w, src);
+        const float gc = c < 2 ? (c == 0 ? gx : gy) : (c == 2 ? gz : gw);
+        float wb[T.kBuckets], ws[2] = {1.f, 1.f}, wt[2] = {1.f, 1.f};
+        if constexpr (FILTER == RT_QUADRILINEAR) {
+            const float u = __shfl_sync(kAll, L.u.w, src), v = __shfl_sync(kAll, L.v.w, src);
+            wb[0] = (1.f - u) * (1.f - v);
+            wb[1] = u * (1.f - v);
+            wb[2] = (1.f - u) * v;
+            wb[3] = u * v;
+        } else {
+            wb[0] = 1.f;
+        }
+        if constexpr (FILTER != RT_NEAREST) {
+            ws[1] = __shfl_sync(kAll, L.s.w, src);
+            wt[1] = __shfl_sync(kAll, L.t.w, src);
+            ws[0] = 1.f - ws[1];
+            wt[0] = 1.f - wt[1];
+        }
+        int64_t ob[T.kBuckets], ot[T.kTexels];
+#pragma unroll
+        for (int b = 0; b < T.kBuckets; ++b) ob[b] = __shfl_sync(kAll, T.bucket[b], src);
+#pragma unroll
+        for (int k = 0; k < T.kTexels; ++k) ot[k] = __shfl_sync(kAll, T.texel[k], src);
+#ifdef RADTEX_CHECKED
+        const int64_t extent = __shfl_sync(kAll, has ? d.extent : (int64_t)0, src);
+#endif
+        if (!hr) continue;
+        auto add = [&](int b, int k, unsigned long long v) {
+            int64_t idx = ob[b] + ot[k];
+#ifdef RADTEX_CHECKED
+            if (idx < 0 || idx >= extent) {
+                atomicOr(status, ST_BOUNDS);
+                idx = 0;
+            }
+#endif
+            atomicAdd(reinterpret_cast<unsigned long long*>(base + 32 * idx), v);
+        };
+        // the weights lie in [0, 1], so |g| decides for every contribution
+        const bool small = fabsf(gc) <= kFixedSmall;
+        float w[T.kBuckets][T.kTexels];
+#pragma unroll
+        for (int b = 0; b < T.kBuckets; ++b)
+#pragma unroll
+            for (int k = 0; k < T.kTexels; ++k) w[b][k] = wb[b] * ws[k & 1] * wt[k >> 1];
+        if (small) {
+#pragma unroll
+            for (int b = 0; b < T.kBuckets; ++b)
+#pragma unroll
+                for (int k = 0; k < T.kTexels; ++k)
+                    if (w[b][k] != 0.f) add(b, k, to_fixed_small(w[b][k] * gc));
+        } else {
+#pragma unroll
+            for (int b = 0; b < T.kBuckets; ++b)
+#pragma unroll
+                for (int k = 0; k < T.kTexels; ++k)
+                    if (w[b][k] != 0.f) add(b, k, to_fixed_any(w[b][k] * gc));
+        }
+    }
 }
 
 // The weights a lane whose axis has taps pk0, pk0 + 1 and weight pw (of pk0 + 1)
@@ -47,84 +188,68 @@ __device__ __forceinline__ void partner_axis_weights(int k0, int pk0, float pw, 
 // texel-gradient contributions w_tap g of a lookup: planes pl[k] (k = (s0,t0)
 // (s1,t0) (s0,t1) (s1,t1)), spatial offsets o[b] (b = (u0,v0) (u1,v0) (u0,v1)
 // (u1,v1)).
-template <bool DET>
 __device__ __forceinline__ void reduce_quadrilinear_taps(const TexDesc& d, const Lookup<RT_QUADRILINEAR>& L,
                                                          const int64_t (&pl)[4], const int (&o)[4], float4 g,
                                                          void* grad) {
     const float wu[2] = {1.f - L.u.w, L.u.w}, wv[2] = {1.f - L.v.w, L.v.w};
     const float ws[2] = {1.f - L.s.w, L.s.w}, wt[2] = {1.f - L.t.w, L.t.w};
-    if (DET) {
-        if (grad) {
+    // Neighbouring fragments often update the same texels: lanes 2m and
+    // 2m + 1 (horizontal neighbours on screen) exchange, once per fragment,
+    // their texture's addressing (gradient buffer, plane size, width, n,
+    // layout), their four axes' floors k0 and weights, and dL/dout.  Each
+    // lane then knows the other's weight on each of its own taps -- the same
+    // tap or one a bucket or texel over -- as the same product of the same
+    // axis weights the other lane forms, so both decide alike: for a texel
+    // both reduce into, the even lane adds the odd lane's contribution to its
+    // own and issues one reduction, and the odd lane issues none.  Only pairs
+    // whose four axes each have the two taps k0, k0 + 1 merge (not at a
+    // clamped edge or a wrapped seam).  A lane without a gradient buffer
+    // leaves before the exchange (its partner sees it inactive).
+    if (!grad) return;
+    const unsigned active = __activemask();
+    const int lane = threadIdx.x & 31;
+    const bool partner = (active >> (lane ^ 1)) & 1u;
+    const bool plain = L.u.k1 == L.u.k0 + 1 && L.v.k1 == L.v.k0 + 1 && L.s.k1 == L.s.k0 + 1 &&
+                       L.t.k1 == L.t.k0 + 1 && d.plane < ((int64_t)1 << 32) && d.W < (1 << 17) && d.n < 256;
+    // the texel index of given coordinates depends on (plane, W, n, layout) only
+    // (the layouts are 0 to 3)
+    const uint64_t gp = (uint64_t)grad;
+    const unsigned geo = plain ? ((unsigned)d.W | ((unsigned)d.n << 17) | ((unsigned)(d.layout & 3) << 25))
+                               : (0x80000000u | (unsigned)lane);  // matches no other lane
+    const unsigned id[4] = {(unsigned)gp, (unsigned)(gp >> 32), (unsigned)d.plane, geo};
+    bool merge = partner;
 #pragma unroll
-            for (int b = 0; b < 4; ++b)
+    for (int m = 0; m < 4; ++m) merge &= __shfl_xor_sync(active, id[m], 1) == id[m];
+    const int pk[4] = {__shfl_xor_sync(active, L.u.k0, 1), __shfl_xor_sync(active, L.v.k0, 1),
+                       __shfl_xor_sync(active, L.s.k0, 1), __shfl_xor_sync(active, L.t.k0, 1)};
+    const float pwk[4] = {__shfl_xor_sync(active, L.u.w, 1), __shfl_xor_sync(active, L.v.w, 1),
+                          __shfl_xor_sync(active, L.s.w, 1), __shfl_xor_sync(active, L.t.w, 1)};
+    const float4 pg = make_float4(__shfl_xor_sync(active, g.x, 1), __shfl_xor_sync(active, g.y, 1),
+                                  __shfl_xor_sync(active, g.z, 1), __shfl_xor_sync(active, g.w, 1));
+    // the partner's weight on this lane's coordinates k0 and k0 + 1 of each axis
+    float pu[2], pv[2], ps[2], pt[2];
+    partner_axis_weights(L.u.k0, pk[0], pwk[0], pu);
+    partner_axis_weights(L.v.k0, pk[1], pwk[1], pv);
+    partner_axis_weights(L.s.k0, pk[2], pwk[2], ps);
+    partner_axis_weights(L.t.k0, pk[3], pwk[3], pt);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float w = wu[b & 1] * wv[b >> 1] * ws[k & 1] * wt[k >> 1];
-                    if (w == 0.f) continue;
-                    const int64_t idx = checked_texel(d, pl[k] + o[b]);
-                    red_add_fixed4(static_cast<unsigned long long*>(grad) + 4 * idx,
-                                   make_float4(w * g.x, w * g.y, w * g.z, w * g.w));
-                }
-        }
-    } else {
-        // Neighbouring fragments often update the same texels: lanes 2m and
-        // 2m + 1 (horizontal neighbours on screen) exchange, once per fragment,
-        // their texture's addressing (gradient buffer, plane size, width, n,
-        // layout), their four axes' floors k0 and weights, and dL/dout.  Each
-        // lane then knows the other's weight on each of its own taps -- the same
-        // tap or one a bucket or texel over -- as the same product of the same
-        // axis weights the other lane forms, so both decide alike: for a texel
-        // both reduce into, the even lane adds the odd lane's contribution to its
-        // own and issues one reduction, and the odd lane issues none.  Only pairs
-        // whose four axes each have the two taps k0, k0 + 1 merge (not at a
-        // clamped edge or a wrapped seam).  A lane without a gradient buffer
-        // leaves before the exchange (its partner sees it inactive).
-        if (!grad) return;
-        const unsigned active = __activemask();
-        const int lane = threadIdx.x & 31;
-        const bool partner = (active >> (lane ^ 1)) & 1u;
-        const bool plain = L.u.k1 == L.u.k0 + 1 && L.v.k1 == L.v.k0 + 1 && L.s.k1 == L.s.k0 + 1 &&
-                           L.t.k1 == L.t.k0 + 1 && d.plane < ((int64_t)1 << 32) && d.W < (1 << 17) && d.n < 256;
-        // the texel index of given coordinates depends on (plane, W, n, layout) only
-        // (the layouts are 0 to 3)
-        const uint64_t gp = (uint64_t)grad;
-        const unsigned geo = plain ? ((unsigned)d.W | ((unsigned)d.n << 17) | ((unsigned)(d.layout & 3) << 25))
-                                   : (0x80000000u | (unsigned)lane);  // matches no other lane
-        const unsigned id[4] = {(unsigned)gp, (unsigned)(gp >> 32), (unsigned)d.plane, geo};
-        bool merge = partner;
+    for (int b = 0; b < 4; ++b)
 #pragma unroll
-        for (int m = 0; m < 4; ++m) merge &= __shfl_xor_sync(active, id[m], 1) == id[m];
-        const int pk[4] = {__shfl_xor_sync(active, L.u.k0, 1), __shfl_xor_sync(active, L.v.k0, 1),
-                           __shfl_xor_sync(active, L.s.k0, 1), __shfl_xor_sync(active, L.t.k0, 1)};
-        const float pwk[4] = {__shfl_xor_sync(active, L.u.w, 1), __shfl_xor_sync(active, L.v.w, 1),
-                              __shfl_xor_sync(active, L.s.w, 1), __shfl_xor_sync(active, L.t.w, 1)};
-        const float4 pg = make_float4(__shfl_xor_sync(active, g.x, 1), __shfl_xor_sync(active, g.y, 1),
-                                      __shfl_xor_sync(active, g.z, 1), __shfl_xor_sync(active, g.w, 1));
-        // the partner's weight on this lane's coordinates k0 and k0 + 1 of each axis
-        float pu[2], pv[2], ps[2], pt[2];
-        partner_axis_weights(L.u.k0, pk[0], pwk[0], pu);
-        partner_axis_weights(L.v.k0, pk[1], pwk[1], pv);
-        partner_axis_weights(L.s.k0, pk[2], pwk[2], ps);
-        partner_axis_weights(L.t.k0, pk[3], pwk[3], pt);
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float w = wu[b & 1] * wv[b >> 1] * ws[k & 1] * wt[k >> 1];
-                if (w == 0.f) continue;
-                const float pw = pu[b & 1] * pv[b >> 1] * ps[k & 1] * pt[k >> 1];
-                const bool shared = merge && pw != 0.f;
-                if (shared && (lane & 1)) continue;  // the even lane reduces it for both
-                float4 c = make_float4(w * g.x, w * g.y, w * g.z, w * g.w);
-                if (shared) {
-                    c.x += pw * pg.x;
-                    c.y += pw * pg.y;
-                    c.z += pw * pg.z;
-                    c.w += pw * pg.w;
-                }
-                red_add_v4(static_cast<float*>(grad) + 4 * checked_texel(d, pl[k] + o[b]), c);
+        for (int k = 0; k < 4; ++k) {
+            const float w = wu[b & 1] * wv[b >> 1] * ws[k & 1] * wt[k >> 1];
+            if (w == 0.f) continue;
+            const float pw = pu[b & 1] * pv[b >> 1] * ps[k & 1] * pt[k >> 1];
+            const bool shared = merge && pw != 0.f;
+            if (shared && (lane & 1)) continue;  // the even lane reduces it for both
+            float4 c = make_float4(w * g.x, w * g.y, w * g.z, w * g.w);
+            if (shared) {
+                c.x += pw * pg.x;
+                c.y += pw * pg.y;
+                c.z += pw * pg.z;
+                c.w += pw * pg.w;
             }
-    }
+            red_add_v4(static_cast<float*>(grad) + 4 * checked_texel(d, pl[k] + o[b]), c);
+        }
 }
 
 // UV and in-bucket coordinate gradients of a quadrilinear lookup from its 16
@@ -160,13 +285,13 @@ __device__ __forceinline__ CoordGrad quad_coord_grads(const Lookup<RT_QUADRILINE
     return cg;
 }
 
-template <int FMT, int LAYOUT, bool DET>
+template <int FMT, int LAYOUT>
 __device__ __forceinline__ CoordGrad backward_quadrilinear_planes(const TexDesc& d, const Lookup<RT_QUADRILINEAR>& L,
                                                                   float4 g, void* grad, bool coord_grads) {
     int64_t pl[4];  // (s0,t0) (s1,t0) (s0,t1) (s1,t1)
     int o[4];       // (u0,v0) (u1,v0) (u0,v1) (u1,v1)
     quad_tap_addresses<LAYOUT>(d, L.u, L.v, L.s, L.t, pl, o);
-    reduce_quadrilinear_taps<DET>(d, L, pl, o, g, grad);
+    reduce_quadrilinear_taps(d, L, pl, o, g, grad);
     if (!coord_grads) return CoordGrad{0.f, 0.f, 0.f, 0.f};
     return quad_coord_grads(L, g, [&](int b, int k) {
         const float sc = FMT == RT_E4M3_BUCKET_SCALE ? __ldg(d.scale + o[b]) : 1.0f;
@@ -174,7 +299,7 @@ __device__ __forceinline__ CoordGrad backward_quadrilinear_planes(const TexDesc&
     });
 }
 
-template <int FILTER, int FMT, int LAYOUT, bool DET>
+template <int FILTER, int FMT, int LAYOUT>
 __device__ __forceinline__ CoordGrad backward_taps(const TexDesc& d, const Lookup<FILTER>& L, float4 g, void* grad,
                                                    bool coord_grads) {
     CoordGrad cg = {0.f, 0.f, 0.f, 0.f};
@@ -192,10 +317,7 @@ __device__ __forceinline__ CoordGrad backward_taps(const TexDesc& d, const Looku
                         int64_t idx = texel_index<LAYOUT>(d, a ? L.u.k1 : L.u.k0, b ? L.v.k1 : L.v.k0,
                                                           p ? L.s.k1 : L.s.k0, q ? L.t.k1 : L.t.k0);
                         const float4 c = make_float4(w * g.x, w * g.y, w * g.z, w * g.w);
-                        if (DET)
-                            red_add_fixed4(static_cast<unsigned long long*>(grad) + 4 * idx, c);
-                        else
-                            red_add_v4(static_cast<float*>(grad) + 4 * idx, c);
+                        red_add_v4(static_cast<float*>(grad) + 4 * idx, c);
                     }
     }
     if (FILTER == RT_NEAREST || !coord_grads) return cg;
@@ -241,42 +363,42 @@ __device__ __forceinline__ CoordGrad backward_taps(const TexDesc& d, const Looku
     }
 }
 
-template <int FILTER, int FMT, int LAYOUT, bool DET>
+template <int FILTER, int FMT, int LAYOUT>
 __device__ __forceinline__ CoordGrad backward_layout(const TexDesc& d, const Lookup<FILTER>& L, float4 g, void* grad,
                                                      bool coord_grads) {
     if constexpr (FILTER == RT_QUADRILINEAR && LAYOUT != RT_LAYOUT_ATLAS)
-        return backward_quadrilinear_planes<FMT, LAYOUT, DET>(d, L, g, grad, coord_grads);
+        return backward_quadrilinear_planes<FMT, LAYOUT>(d, L, g, grad, coord_grads);
     else
-        return backward_taps<FILTER, FMT, LAYOUT, DET>(d, L, g, grad, coord_grads);
+        return backward_taps<FILTER, FMT, LAYOUT>(d, L, g, grad, coord_grads);
 }
 
-template <int FILTER, int FMT, bool DET>
+template <int FILTER, int FMT>
 __device__ __forceinline__ CoordGrad backward_dense(const TexDesc& d, const Lookup<FILTER>& L, float4 g, void* grad,
                                                     bool coord_grads) {
     // as filter_dense: owned textures QUADS (bits PLANES), borrowed FP32 buffers QUADS or PLANES
-    if (d.layout == kLayoutPalette) return backward_layout<FILTER, FMT, kLayoutPalette, DET>(d, L, g, grad, coord_grads);
-    if (FMT == RT_BIT1) return backward_layout<FILTER, FMT, RT_LAYOUT_PLANES, DET>(d, L, g, grad, coord_grads);
+    if (d.layout == kLayoutPalette) return backward_layout<FILTER, FMT, kLayoutPalette>(d, L, g, grad, coord_grads);
+    if (FMT == RT_BIT1) return backward_layout<FILTER, FMT, RT_LAYOUT_PLANES>(d, L, g, grad, coord_grads);
     if (FMT != RT_F32 || d.layout == RT_LAYOUT_QUADS)
-        return backward_layout<FILTER, FMT, RT_LAYOUT_QUADS, DET>(d, L, g, grad, coord_grads);
-    return backward_layout<FILTER, FMT, RT_LAYOUT_PLANES, DET>(d, L, g, grad, coord_grads);
+        return backward_layout<FILTER, FMT, RT_LAYOUT_QUADS>(d, L, g, grad, coord_grads);
+    return backward_layout<FILTER, FMT, RT_LAYOUT_PLANES>(d, L, g, grad, coord_grads);
 }
 
-template <int FILTER, bool DET>
+template <int FILTER>
 __device__ __forceinline__ CoordGrad backward_any(const TexDesc& d, const Lookup<FILTER>& L, float4 g, void* grad,
                                                   bool coord_grads) {
     switch (d.fmt) {
         case RT_F16:
-            return backward_dense<FILTER, RT_F16, DET>(d, L, g, grad, coord_grads);
+            return backward_dense<FILTER, RT_F16>(d, L, g, grad, coord_grads);
         case RT_BF16:
-            return backward_dense<FILTER, RT_BF16, DET>(d, L, g, grad, coord_grads);
+            return backward_dense<FILTER, RT_BF16>(d, L, g, grad, coord_grads);
         case RT_BIT1:  // no texel gradients (rejected on the host); coordinate gradients only
-            return backward_dense<FILTER, RT_BIT1, DET>(d, L, g, nullptr, coord_grads);
+            return backward_dense<FILTER, RT_BIT1>(d, L, g, nullptr, coord_grads);
         case RT_E4M3_BUCKET_SCALE:
-            return backward_dense<FILTER, RT_E4M3_BUCKET_SCALE, DET>(d, L, g, grad, coord_grads);
+            return backward_dense<FILTER, RT_E4M3_BUCKET_SCALE>(d, L, g, grad, coord_grads);
         default:
             if (d.layout == RT_LAYOUT_ATLAS)
-                return backward_layout<FILTER, RT_F32, RT_LAYOUT_ATLAS, DET>(d, L, g, grad, coord_grads);
-            return backward_dense<FILTER, RT_F32, DET>(d, L, g, grad, coord_grads);
+                return backward_layout<FILTER, RT_F32, RT_LAYOUT_ATLAS>(d, L, g, grad, coord_grads);
+            return backward_dense<FILTER, RT_F32>(d, L, g, grad, coord_grads);
     }
 }
 
@@ -330,13 +452,13 @@ __device__ __forceinline__ float2 uv_grad(const TexDesc& d, float u, float v, fl
 }
 
 // SPEC as in filter_spec: one format for every object, or -1 (dispatch).
-template <int FILTER, bool DET, int SPEC>
+template <int FILTER, int SPEC>
 __device__ __forceinline__ CoordGrad backward_spec(const TexDesc& d, const Lookup<FILTER>& L, float4 g, void* grad,
                                                    bool coord_grads) {
     if constexpr (SPEC < 0)
-        return backward_any<FILTER, DET>(d, L, g, grad, coord_grads);
+        return backward_any<FILTER>(d, L, g, grad, coord_grads);
     else
-        return backward_layout<FILTER, SPEC, RT_LAYOUT_QUADS, DET>(d, L, g, grad, coord_grads);
+        return backward_layout<FILTER, SPEC, RT_LAYOUT_QUADS>(d, L, g, grad, coord_grads);
 }
 
 // UV and direction gradients of one fragment from its weight-coordinate
