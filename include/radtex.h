@@ -219,6 +219,14 @@ int64_t rt_kmeans_tc_scratch_bytes(int32_t w, int32_t h, int32_t n, int32_t K);
 rt_status rt_kmeans_assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
                               float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream);
 
+/* rt_kmeans_assign_tc again with other centroids: `scratch` still holds what an
+ * earlier rt_kmeans_assign_tc of the same texture left in it (same object,
+ * texels unchanged since, same K and scratch, ordered before this call), so the
+ * bucket vectors are not converted again.  The Lloyd steps of one encoding call
+ * it after the first assignment. */
+rt_status rt_kmeans_reassign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
+                                float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream);
+
 /* The number of polls (each followed by a 32 ns sleep) after which a bounded
  * wait of the library's kernels -- the mbarrier waits of the tensor-core
  * k-means assignment's pipeline -- gives up: the kernel then raises

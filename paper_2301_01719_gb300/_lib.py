@@ -79,6 +79,7 @@ SIGNATURES = {
     "rt_kmeans_init": (_I32, [_P, _I32, _I32, _P, _P, _P]),
     "rt_kmeans_tc_scratch_bytes": (_I64, [_I32, _I32, _I32, _I32]),
     "rt_kmeans_assign_tc": (_I32, [_P, _I32, _I32, _P, _P, _P, _P, _I64, _P]),
+    "rt_kmeans_reassign_tc": (_I32, [_P, _I32, _I32, _P, _P, _P, _P, _I64, _P]),
     "rt_kmeans_assign": (_I32, [_P, _I32, _I32, _P, _P, _P, _P]),
     "rt_kmeans_update": (_I32, [_P, _I32, _I32, _P, _P, _P, _P]),
     "rt_shade": (_I32, [_P, _P, _P, _P, _I64, _I32, _P, _P]),

@@ -189,6 +189,18 @@ def rt_kmeans_assign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Tens
     return (index, dist) if want_dist else index
 
 
+def rt_kmeans_reassign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Tensor, index: torch.Tensor,
+                          dist: torch.Tensor | None, scratch: TcScratch, stream=None) -> torch.Tensor:
+    """rt_kmeans_assign_tc with other centroids, on the scratch that an earlier call of it on the
+    same (unchanged) texture left: the bucket vectors are not converted again."""
+    _check(centroids, "centroids", torch.float32, 4)
+    if centroids.numel() != K * rt_texture_info(ctx, obj_id)["n"] ** 2 * 4:
+        raise ValueError("centroids must hold K x n x n x 4 values")
+    _lib.call("rt_kmeans_reassign_tc", ctx.handle, int(obj_id), int(K), _ptr(centroids), _ptr(index), _ptr(dist),
+              ctypes.c_void_p(scratch.ptr), int(scratch.nbytes), _stream(stream, centroids.device))
+    return index
+
+
 def rt_kmeans_update(ctx: Context, obj_id: int, K: int, index: torch.Tensor, centroids: torch.Tensor,
                      scratch: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """Centroids <- means of their members (in place); empty centroids are kept."""
@@ -225,19 +237,21 @@ def palette_encode(ctx: Context, obj_id: int, K: int, iterations: int, seed: int
     sse = []
     tc = TcScratch(rt_kmeans_tc_scratch_bytes(info["w"], info["h"], info["n"], K), dev) if tensor_cores else None
 
-    def assign():
-        if tensor_cores:
+    def assign(first):
+        if not tensor_cores:
+            rt_kmeans_assign(ctx, obj_id, K, C, index, dist, stream=stream)
+        elif first:
             rt_kmeans_assign_tc(ctx, obj_id, K, C, index, dist, scratch=tc, stream=stream)
         else:
-            rt_kmeans_assign(ctx, obj_id, K, C, index, dist, stream=stream)
+            rt_kmeans_reassign_tc(ctx, obj_id, K, C, index, dist, tc, stream=stream)
 
-    for _ in range(iterations):
-        assign()
-        sse.append(dist.double().sum())
+    for step in range(iterations):
+        assign(step == 0)
+        sse.append(dist.sum(dtype=torch.float64))
         rt_kmeans_update(ctx, obj_id, K, index, C, scratch, stream=stream)
-    assign()
-    sse.append(dist.double().sum())
-    return C, index, [float(x) for x in sse]
+    assign(iterations == 0)
+    sse.append(dist.sum(dtype=torch.float64))
+    return C, index, torch.stack(sse).tolist()
 
 
 def rt_destroy_texture(ctx: Context, obj_id: int) -> None:

@@ -489,8 +489,8 @@ int64_t rt_kmeans_tc_scratch_bytes(int32_t w, int32_t h, int32_t n, int32_t K) {
     return rt::kmeans_tc_scratch_bytes(w, h, n, K);
 }
 
-rt_status rt_kmeans_assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
-                              float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream) {
+static rt_status assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
+                           float* dist, void* scratch, int64_t scratch_bytes, bool converted, rt_stream_t stream) {
     if (!kmeans_source(ctx, obj_id, K) || !centroids || !aligned16(centroids) || !index || !scratch ||
         (reinterpret_cast<uintptr_t>(scratch) & 1023u) != 0)
         return RT_ERR_INVALID_ARG;
@@ -498,9 +498,19 @@ rt_status rt_kmeans_assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const floa
     if (scratch_bytes < rt::kmeans_tc_scratch_bytes(d.W, d.H, d.n, K)) return RT_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
-    cudaError_t e = rt::launch_kmeans_assign_tc(d, K, centroids, index, dist, scratch, ctx->d_status,
+    cudaError_t e = rt::launch_kmeans_assign_tc(d, K, centroids, index, dist, scratch, converted, ctx->d_status,
                                                 ctx->wait_limit, (cudaStream_t)stream);
     return e == cudaErrorNotSupported ? RT_ERR_UNSUPPORTED : cuda_status(e);
+}
+
+rt_status rt_kmeans_assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
+                              float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream) {
+    return assign_tc(ctx, obj_id, K, centroids, index, dist, scratch, scratch_bytes, false, stream);
+}
+
+rt_status rt_kmeans_reassign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
+                                float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream) {
+    return assign_tc(ctx, obj_id, K, centroids, index, dist, scratch, scratch_bytes, true, stream);
 }
 
 rt_status rt_set_wait_limit(rt_ctx* ctx, uint32_t polls) {
