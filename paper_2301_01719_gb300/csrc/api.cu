@@ -29,6 +29,7 @@ struct rt_ctx {
     long long* det[RT_MAX_OBJECTS];      // fixed-point gradient sums of the deterministic mode
     uint32_t* index[RT_MAX_OBJECTS];     // palette index maps the library copied
     int spec = -1;                       // the format shared by all objects (dense PLANES, clamp), else -1
+    int bits = rt::kBitsNone;            // how the bits are indexed if all objects are bit textures in clamp mode
     uint32_t wait_limit = 0;             // polls of a bounded device wait before it gives up (0: the default)
 };
 
@@ -108,8 +109,24 @@ int table_spec(const rt_ctx* ctx) {
     return spec < 0 ? -1 : spec;
 }
 
+// How the objects' bits are indexed if every object is a bit texture in clamp mode.
+int table_bits(const rt_ctx* ctx) {
+    int bits = rt::kBitsNone;
+    for (int o = 0; o < ctx->n_obj; ++o) {
+        const TexDesc& d = ctx->table[o];
+        if (!d.live) continue;
+        if (d.fmt != RT_BIT1 || d.layout != RT_LAYOUT_PLANES || d.wrap) return rt::kBitsNone;
+        const int need = d.plane * d.n * d.n >= ((int64_t)1 << 32) ? rt::kBitsLarge
+                         : d.plane % 32 != 0                       ? rt::kBitsSmall
+                                                                   : rt::kBitsWords;
+        if (need > bits) bits = need;
+    }
+    return bits;
+}
+
 rt_status upload_table(rt_ctx* ctx) {
     ctx->spec = table_spec(ctx);
+    ctx->bits = table_bits(ctx);
     cudaError_t e = cudaMemcpy(ctx->d_table, ctx->table, sizeof(TexDesc) * RT_MAX_OBJECTS, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     return cuda_status(e);
@@ -740,7 +757,7 @@ rt_status rt_shade_multi(rt_ctx* ctx, const float* uv, const float* dirs, int32_
     if (!out || !aligned16(out)) return RT_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
-    return cuda_status(rt::launch_multi_shade(ctx->d_table, ctx->n_obj, uv, dirs, samples, obj, F, filter, out,
+    return cuda_status(rt::launch_multi_shade(ctx->d_table, ctx->n_obj, uv, dirs, samples, obj, F, filter, ctx->bits, out,
                                               ctx->d_status, (cudaStream_t)stream));
 }
 

@@ -8,6 +8,8 @@
 // a constant texture returns its constant exactly.
 #pragma once
 
+#include <type_traits>
+
 #include "rt_device.cuh"
 
 namespace rt {
@@ -116,6 +118,73 @@ __device__ __forceinline__ float4 filter_taps(const TexDesc& d, const Lookup<FIL
             y[bv] = lerpP(c[0], c[1], wu);
         }
         return toF4(lerpP(y[0], y[1], wv));
+    }
+}
+
+// How the bit textures of a context are indexed: planes of whole words and fewer
+// than 2^32 texels, any planes with fewer than 2^32 texels, or any.
+enum { kBitsNone = 0, kBitsWords = 1, kBitsSmall = 2, kBitsLarge = 3 };
+
+// The value of a lookup in a bit texture (PLANES, clamp), equal in its four
+// channels: the nested lerps of filter_taps on one number.  The two buckets of a
+// row at one in-bucket texel are neighbouring bits, nearly always of one word;
+// the pair is filtered as a packed pair.  With planes of whole words a row lies
+// at the same bit of its word in all four planes.
+template <int FILTER, int KIND>
+__device__ __forceinline__ float filter_bits(const TexDesc& d, const Lookup<FILTER>& L) {
+    using Idx = typename std::conditional<KIND == kBitsLarge, int64_t, uint32_t>::type;
+    const unsigned* words = reinterpret_cast<const unsigned*>(d.base);
+    auto value = [](unsigned bits) { return __uint_as_float((bits & 1u) * 0x3f800000u); };  // 0.0f or 1.0f
+    auto lerpf = [](float a, float b, float w) { return fmaf(w, b - a, a); };
+    const Idx P = (Idx)d.plane, p00 = (Idx)(L.t.k0 * d.n + L.s.k0) * P;
+    const Idx o0 = (Idx)bucket_slot<RT_LAYOUT_PLANES>(d, L.u.k0, L.v.k0);
+    auto texel = [&](Idx o) {
+        const Idx e = (Idx)checked_texel(d, (int64_t)o);
+        return value(__ldg(words + (e >> 5)) >> ((unsigned)e & 31u));
+    };
+    if constexpr (FILTER == RT_NEAREST) return texel(p00 + o0);
+    const Idx ds = (Idx)(L.s.k1 - L.s.k0) * P, dt = (Idx)((L.t.k1 - L.t.k0) * d.n) * P;
+    const Idx pl[4] = {p00, p00 + ds, p00 + dt, p00 + dt + ds};
+    if constexpr (FILTER == RT_ANGULAR_BILINEAR) {
+        return lerpf(lerpf(texel(pl[0] + o0), texel(pl[1] + o0), L.s.w),
+                     lerpf(texel(pl[2] + o0), texel(pl[3] + o0), L.s.w), L.t.w);
+    } else {
+        const Idx o1 = (Idx)bucket_slot<RT_LAYOUT_PLANES>(d, L.u.k0, L.v.k1);
+        const unsigned u1 = (unsigned)(L.u.k1 - L.u.k0);  // 0 (clamped) or 1
+        const f32x2 ws = pack2(L.s.w, L.s.w), wt = pack2(L.t.w, L.t.w);
+        float row[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const Idx o = r ? o1 : o0;
+            unsigned lo[4], hi[4], sh[4];  // the word of the first bucket's bit, the next one's, the bit
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const Idx a = (Idx)checked_texel(d, (int64_t)(pl[k] + o));
+                if (KIND == kBitsWords) {
+                    lo[k] = __ldg(words + ((pl[k] >> 5) + (o >> 5)));
+                    sh[k] = (unsigned)o & 31u;
+                } else {
+                    lo[k] = __ldg(words + (a >> 5));
+                    sh[k] = (unsigned)a & 31u;
+                }
+                hi[k] = lo[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (u1 == 1u && sh[k] == 31u) {
+                    const Idx b = (Idx)checked_texel(d, (int64_t)(pl[k] + o + 1));
+                    hi[k] = __ldg(words + (b >> 5));
+                }
+            f32x2 q[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const unsigned x = __funnelshift_r(lo[k], hi[k], sh[k]);  // the two bits, lowest first
+                q[k] = pack2(value(x), value(x >> u1));
+            }
+            const float2 c = unpack2(lerp2(lerp2(q[0], q[1], ws), lerp2(q[2], q[3], ws), wt));
+            row[r] = lerpf(c.x, c.y, L.u.w);
+        }
+        return lerpf(row[0], row[1], L.v.w);
     }
 }
 

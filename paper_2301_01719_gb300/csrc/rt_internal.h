@@ -87,8 +87,9 @@ cudaError_t launch_read(const void* src, int src_layout, const float* scale, int
                         int dst_layout, void* dst, float* scale_dst, cudaStream_t stream);
 cudaError_t launch_bake_shadow(const rt_bake_scene& S, int surface, void* dst, int W, int H, int n,
                                cudaStream_t stream);
+// bits: kBitsNone, or how the objects are indexed if all are bit textures in clamp mode.
 cudaError_t launch_multi_shade(const TexDesc* table, int n_obj, const float* uv, const float* dirs, int S,
-                               const int32_t* obj, int64_t F, int filter, float* out, unsigned* status,
+                               const int32_t* obj, int64_t F, int filter, int bits, float* out, unsigned* status,
                                cudaStream_t stream);
 // World-space kernels: T is flat_tiling() for the flat stream, or a screen tiling.
 cudaError_t launch_world_shade(const TexDesc* table, int n_obj, const float* uv, const float* dir, const float* nrm,

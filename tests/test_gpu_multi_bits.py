@@ -1,0 +1,92 @@
+"""rt_shade_multi on contexts of bit textures alone against the dispatching kernels, which run as
+soon as the context holds an object of another format: the same colours bit for bit, for every
+filter, sample counts that do and do not divide a warp, odd sizes and invalid samples."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from paper_2301_01719_gb300 import api
+
+pytestmark = pytest.mark.gpu
+
+FILTERS = [api.RT_NEAREST, api.RT_ANGULAR_BILINEAR, api.RT_QUADRILINEAR]
+
+
+def _inputs(F, S, seed, objects):
+    rng = np.random.default_rng(seed)
+    uv = rng.uniform(-0.1, 1.1, (F, 2)).astype(np.float32)  # beyond both edges
+    d = rng.standard_normal((F, S, 3)).astype(np.float32)
+    d[..., 2] = np.abs(d[..., 2])
+    d /= np.linalg.norm(d, axis=-1, keepdims=True)
+    obj = rng.integers(-1, objects, F).astype(np.int32)
+    return uv, d, obj
+
+
+def _both(sizes, seed, uv, d, obj, filt, fill=None):
+    """The call on a context of bit textures, then with an FP32 object added: colours and statuses."""
+    got = []
+    with_other = (False, True)
+    for other in with_other:
+        ctx = api.Context(0)
+        for k, (w, h, n) in enumerate(sizes):
+            if fill is None:
+                src = torch.rand(api.layout_shape(api.RT_LAYOUT_PLANES, w, h, n),
+                                 generator=torch.Generator("cuda").manual_seed(seed + k), device="cuda")
+                api.rt_create_texture(ctx, w, h, n, api.RT_BIT1, api.RT_LAYOUT_PLANES, src)
+            else:
+                fill(ctx, api.rt_create_texture(ctx, w, h, n, api.RT_BIT1))
+        if other:
+            api.rt_create_texture(ctx, 1, 1, 1, api.RT_F32)
+        out = api.rt_shade_multi(ctx, torch.from_numpy(uv).cuda(), torch.from_numpy(d).cuda(),
+                                 torch.from_numpy(obj).cuda(), filt)
+        got.append((out.cpu().numpy(), api.rt_get_error(ctx)))
+        ctx.close()
+    return got
+
+
+@pytest.mark.parametrize("filt", FILTERS)
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 5, 7, 8, 11, 16, 31, 32, 33])
+@pytest.mark.parametrize("sizes", [[(37, 23, 5), (64, 32, 8), (1, 1, 1)],  # planes of whole words or not,
+                                   [(64, 32, 8), (37, 32, 3), (1, 32, 2)]])  # and all of whole words
+def test_bit_contexts_match_the_dispatching_kernels(filt, S, sizes):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    uv, d, obj = _inputs(1003, S, S, 3)
+    (a, ea), (b, eb) = _both(sizes, 5, uv, d, obj, filt)
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+    assert ea == eb == api.RT_OK and a.any() and not a[obj < 0].any()
+
+
+@pytest.mark.parametrize("S", [3, 4])
+def test_invalid_samples_zero_their_fragment(S):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    for where, status in (("direction", api.RT_ERR_NONFINITE), ("uv", api.RT_ERR_NONFINITE),
+                          ("object", api.RT_ERR_BAD_OBJ_ID)):
+        uv, d, obj = _inputs(257, S, 9, 1)
+        obj[:] = 0
+        if where == "direction":
+            d[100, S - 1, 1] = np.nan
+        elif where == "uv":
+            uv[100, 0] = np.inf
+        else:
+            obj[100] = 900
+        (a, ea), (b, eb) = _both([(16, 16, 4)], 6, uv, d, obj, api.RT_QUADRILINEAR)
+        np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+        assert ea == eb == status and not a[100].any()
+
+
+def test_textures_of_2_to_the_32_texels_take_64_bit_indices():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    uv, d, obj = _inputs(40001, 4, 3, 1)
+    obj[:] = 0
+    scene = synth.bake_scene(11)
+
+    def fill(ctx, oid):
+        api.rt_bake_shadow(ctx, oid, api.RT_SURFACE_PLANE, scene)
+
+    (a, ea), (b, eb) = _both([(65536, 16384, 2)], 0, uv, d, obj, api.RT_QUADRILINEAR, fill)
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+    assert ea == eb == api.RT_OK and 0.0 < a.mean() < 1.0
