@@ -60,8 +60,7 @@ SIGNATURES = {
     "rt_context_destroy": (None, [_P]),
     "rt_create_texture": (_I32, [_P, _I32, _I32, _I32, _I32, _I32, _P, _I32, ctypes.POINTER(_I32)]),
     "rt_destroy_texture": (_I32, [_P, _I32]),
-    "rt_texture_info": (_I32, [_P, _I32, ctypes.POINTER(_I32), ctypes.POINTER(_I32), ctypes.POINTER(_I32),
-                               ctypes.POINTER(_I32), ctypes.POINTER(_I32), ctypes.POINTER(_I64)]),
+    "rt_texture_info": (_I32, [_P, _I32, _P, _P, _P, _P, _P, _P]),
     "rt_read_texture": (_I32, [_P, _I32, _I32, _P, _P, _P]),
     "rt_fill_bucket_lobes": (_I32, [_P, _I32, _P, _P]),
     "rt_bake": (_I32, [_P, _I32, _I32, _P, _P]),
@@ -152,5 +151,13 @@ def check(fn: str, status: int) -> None:
         raise RadtexError(fn, status)
 
 
+_entry = {}  # the library's functions by name, once it is loaded
+
+
 def call(name: str, *args) -> None:
-    check(name, getattr(lib(), name)(*args))
+    fn = _entry.get(name)
+    if fn is None:
+        fn = _entry[name] = getattr(lib(), name)
+    status = fn(*args)
+    if status != RT_OK:
+        raise RadtexError(name, status)

@@ -8,6 +8,7 @@ tensors' device.  All the work happens in the library's CUDA kernels.
 from __future__ import annotations
 
 import ctypes
+import math
 
 import numpy as np
 import torch
@@ -30,20 +31,19 @@ FILTER_NAMES = {"nearest": RT_NEAREST, "angular_bilinear": RT_ANGULAR_BILINEAR, 
 
 
 def _ptr(t: torch.Tensor | None):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream, device) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream(device)
-    handle = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
-    return ctypes.c_void_p(handle)
+def _stream(stream, device) -> int:
+    if stream is None:  # torch.cuda.current_stream(device).cuda_stream without the Stream object (2 us)
+        return torch._C._cuda_getCurrentRawStream(device.index)
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(t: torch.Tensor, name: str, dtype, last_dim: int | None = None):
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -185,7 +185,7 @@ def rt_kmeans_assign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Tens
     if scratch is None:
         scratch = TcScratch(rt_kmeans_tc_scratch_bytes(info["w"], info["h"], info["n"], K), dev)
     _lib.call("rt_kmeans_assign_tc", ctx.handle, int(obj_id), int(K), _ptr(centroids), _ptr(index), _ptr(dist),
-              ctypes.c_void_p(scratch.ptr), int(scratch.nbytes), _stream(stream, dev))
+              scratch.ptr, int(scratch.nbytes), _stream(stream, dev))
     return (index, dist) if want_dist else index
 
 
@@ -197,7 +197,7 @@ def rt_kmeans_reassign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Te
     if centroids.numel() != K * rt_texture_info(ctx, obj_id)["n"] ** 2 * 4:
         raise ValueError("centroids must hold K x n x n x 4 values")
     _lib.call("rt_kmeans_reassign_tc", ctx.handle, int(obj_id), int(K), _ptr(centroids), _ptr(index), _ptr(dist),
-              ctypes.c_void_p(scratch.ptr), int(scratch.nbytes), _stream(stream, centroids.device))
+              scratch.ptr, int(scratch.nbytes), _stream(stream, centroids.device))
     return index
 
 
@@ -258,11 +258,20 @@ def rt_destroy_texture(ctx: Context, obj_id: int) -> None:
     _lib.call("rt_destroy_texture", ctx.handle, int(obj_id))
 
 
+_Info = ctypes.c_int32 * 5
+
+
+def _texture_info(ctx: Context, obj_id: int, nbytes=None) -> tuple:
+    """(w, h, n, storage, layout)."""
+    v = _Info()
+    _lib.call("rt_texture_info", ctx.handle, int(obj_id), v, ctypes.byref(v, 4), ctypes.byref(v, 8),
+              ctypes.byref(v, 12), ctypes.byref(v, 16), nbytes)
+    return tuple(v)
+
+
 def rt_texture_info(ctx: Context, obj_id: int) -> dict:
-    vals = [ctypes.c_int32() for _ in range(5)]
     nbytes = ctypes.c_int64()
-    _lib.call("rt_texture_info", ctx.handle, int(obj_id), *[ctypes.byref(v) for v in vals], ctypes.byref(nbytes))
-    w, h, n, storage, layout = (v.value for v in vals)
+    w, h, n, storage, layout = _texture_info(ctx, obj_id, ctypes.byref(nbytes))
     return {"w": w, "h": h, "n": n, "storage": storage, "layout": layout, "bytes": nbytes.value}
 
 
@@ -283,17 +292,16 @@ def _padded(layout: int, w: int, h: int) -> bool:
 
 
 def layout_numel(layout: int, w: int, h: int, n: int) -> int:
-    return int(np.prod(layout_shape(layout, w, h, n)))
+    return math.prod(layout_shape(layout, w, h, n))
 
 
 def storage_numel(ctx: Context, obj_id: int) -> int:
     """Values (4 per texel) of a buffer in the object's storage layout: its texel
     gradients (rt_shade_backward's dL_dtex) and its stored codes."""
-    info = rt_texture_info(ctx, obj_id)
-    K = rt_palette_size(ctx, obj_id)
-    if K:
-        return K * info["n"] ** 2 * 4
-    return layout_numel(info["layout"], info["w"], info["h"], info["n"])
+    w, h, n, _, layout = _texture_info(ctx, obj_id)
+    if layout == RT_LAYOUT_PALETTE:
+        return rt_palette_size(ctx, obj_id) * n * n * 4
+    return layout_numel(layout, w, h, n)
 
 
 def rt_read_texture(ctx: Context, obj_id: int, dst_layout: int = RT_LAYOUT_ATLAS, stream=None):
