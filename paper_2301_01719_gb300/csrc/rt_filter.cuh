@@ -231,10 +231,9 @@ __device__ __forceinline__ float4 filter_spec(const TexDesc& d, const Lookup<FIL
 // G-buffer staging.  Kernels that walk fragments are persistent: each warp
 // takes 32-fragment chunks c, c + (warps in the grid), ...  and double-buffers
 // them in its own slice of shared memory.  While the warp filters chunk c, the
-// G-buffer of its next chunk (uv 256 B, dir 384 B, obj 128 B, and optionally a
-// 16-byte-per-fragment extra stream such as dL/dout) is already in flight with
-// 16-byte cp.async copies that bypass L1 -- so the DRAM latency of the
-// G-buffer overlaps the texel gather, and no block-wide barrier is needed.
+// G-buffer of its next chunk is already in flight with 16-byte cp.async copies
+// that bypass L1 -- so the DRAM latency of the G-buffer overlaps the texel
+// gather, and no block-wide barrier is needed.
 // Only __syncwarp orders the warp's own copies and reads.
 //
 // A chunk is either 32 consecutive fragments of the flat stream (rt_shade), or
@@ -285,16 +284,16 @@ struct Tiling {
 };
 
 // A warp's G-buffer buffers: the chunk being processed plus STAGES - 1
-// prefetched ones.
-// NRM adds a second three-float stream (the per-fragment normal of the
-// world-space lookup), staged like dir.
+// prefetched ones.  A chunk is 24 pieces of 16 bytes of dir, 16 of uv and 8 of
+// obj, in fragment order, then optionally a 16-byte-per-fragment extra stream
+// such as dL/dout and (NRM) a second three-float stream, the normal of the
+// world-space lookup.
 template <bool EXTRA, int STAGES = 2, bool NRM = false>
-struct WarpStage {
-    float uv[STAGES][2 * kChunk];
-    float dir[STAGES][3 * kChunk];
-    int obj[STAGES][kChunk];
-    float4 extra[EXTRA ? STAGES : 1][EXTRA ? kChunk : 1];
-    float nrm[NRM ? STAGES : 1][NRM ? 3 * kChunk : 1];
+struct __align__(16) WarpStage {
+    static constexpr int kDir = 0, kUv = 12 * kChunk, kObj = 20 * kChunk, kExtra = 24 * kChunk;
+    static constexpr int kNrm = kExtra + (EXTRA ? 16 * kChunk : 0);
+    static constexpr int kBytes = kNrm + (NRM ? 12 * kChunk : 0);
+    char b[STAGES][kBytes];
 };
 
 struct Frag {
@@ -303,9 +302,13 @@ struct Frag {
     float nx, ny, nz;  // NRM streams only
 };
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+// Asynchronous copies of BYTES (4 or 8 through L1, 16 past it) to shared address s.
+template <int BYTES>
+__device__ __forceinline__ void cp_async(unsigned s, const void* gmem) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -313,173 +316,203 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Geometry of one chunk: the first fragment of each of its rows, whether the
-// whole chunk can be copied with aligned 16-byte pieces, and this lane's
-// fragment (-1 = none).
-struct ChunkGeom {
-    int64_t row0;    // fragment index of (x0, y0)
-    int64_t pitch;   // fragment stride between rows
-    int tw, th, tw_log2;
+// One chunk: the first fragment of its first row, whether all of it can be
+// copied in aligned 16-byte pieces, and this lane's fragment (-1 = none).
+struct Chunk {
+    int64_t row0;
+    int64_t f;
     bool fast;
-    int64_t f;       // this lane's fragment, -1 outside the frame / stream
 };
 
+// The chunks of one warp, in order.  Tiled: block tiles blockIdx.x,
+// blockIdx.x + gridDim.x, ... in raster order, frame after frame, this warp's
+// tile of each; the step is taken in tile coordinates, so that a chunk costs a
+// few additions and no division.  Flat: 32-fragment runs.
 template <int WARPS, bool TILED>
-__device__ __forceinline__ ChunkGeom chunk_geom(const Tiling& T, int64_t F, int64_t c, int lane) {
-    ChunkGeom g;
-    if (!TILED) {
-        g.row0 = c * kChunk;
-        g.pitch = kChunk;
-        g.tw = kChunk;
-        g.th = 1;
-        g.tw_log2 = 5;
-        g.fast = g.row0 + kChunk <= F;
-        g.f = g.row0 + lane < F ? g.row0 + lane : -1;
+struct ChunkWalk {
+    int tx, ty, view, dx, dy, dv;  // block tile and step (tiled)
+    int wx, wy, lx, ly;            // this warp's tile in the block tile, this lane in the tile
+    int64_t c, dc;                 // chunk and step (flat)
+    int64_t count;                 // chunks left to hand out
+
+    __device__ __forceinline__ ChunkWalk(const Tiling& T, int64_t F, int lane, int w) {
+        if constexpr (TILED) {
+            const uint32_t bt = blockIdx.x, step = gridDim.x;
+            tiles(T, bt, tx, ty, view);
+            tiles(T, step, dx, dy, dv);
+            const int64_t total = (int64_t)T.btx * T.bty * T.views;
+            count = bt < total ? (int64_t)((uint32_t)(total - 1 - bt) / step + 1) : 0;
+            wx = (w & (T.bx - 1)) << T.tw_log2;
+            wy = (w >> T.bx_log2) * T.th;
+            lx = lane & (T.tw - 1);
+            ly = lane >> T.tw_log2;
+        } else {
+            c = (int64_t)blockIdx.x * WARPS + w;
+            dc = (int64_t)gridDim.x * WARPS;
+            const int64_t total = (F + kChunk - 1) / kChunk;
+            count = c < total ? (total - 1 - c) / dc + 1 : 0;
+        }
+    }
+
+    __device__ __forceinline__ static void tiles(const Tiling& T, uint32_t n, int& x, int& y, int& v) {
+        const uint32_t q = T.div_frame.div(n), r = n - q * T.div_frame.d, ry = T.div_btx.div(r);
+        v = (int)q;
+        y = (int)ry;
+        x = (int)(r - ry * T.div_btx.d);
+    }
+
+    // The next chunk (any values once count is used up).
+    __device__ __forceinline__ Chunk next(const Tiling& T, int64_t F, int lane) {
+        Chunk g;
+        if constexpr (TILED) {
+            const int x0 = (tx * T.bx << T.tw_log2) + wx, y0 = ty * (T.by * T.th) + wy;
+            g.row0 = (int64_t)view * T.frame + ((int64_t)y0 * T.W + x0);
+            const bool whole = x0 + T.tw <= T.W && y0 + T.th <= T.H;
+            g.fast = whole && (T.W & 3) == 0;
+            g.f = whole || (x0 + lx < T.W && y0 + ly < T.H) ? g.row0 + (ly * T.W + lx) : -1;
+            tx += dx;
+            ty += dy;
+            view += dv;
+            if (tx >= T.btx) {
+                tx -= T.btx;
+                ++ty;
+            }
+            if (ty >= T.bty) {
+                ty -= T.bty;
+                ++view;
+            }
+        } else {
+            g.row0 = c * kChunk;
+            g.fast = g.row0 + kChunk <= F;
+            g.f = g.row0 + lane < F ? g.row0 + lane : -1;
+            c += dc;
+        }
         return g;
     }
-    // block tile bt, sub-tile w; chunk indices of the tiled walk fit 31 bits
-    const uint32_t cc = (uint32_t)c;
-    const uint32_t bt = cc / WARPS, w = cc % WARPS;
-    const uint32_t view = T.div_frame.div(bt);
-    const uint32_t r = bt - view * T.div_frame.d;
-    const uint32_t tyb = T.div_btx.div(r), txb = r - tyb * T.div_btx.d;
-    const int x0 = (int)((txb * T.bx + (w & (T.bx - 1))) << T.tw_log2);
-    const int y0 = (int)((tyb * T.by + (w >> T.bx_log2)) * T.th);
-    g.tw = T.tw;
-    g.th = T.th;
-    g.tw_log2 = T.tw_log2;
-    g.pitch = T.W;
-    g.row0 = (int64_t)view * T.frame + (int64_t)y0 * T.W + x0;
-    g.fast = (x0 + T.tw <= T.W) && (y0 + T.th <= T.H) && ((T.W & 3) == 0);
-    const int ly = lane >> T.tw_log2, lx = lane & (T.tw - 1);
-    g.f = (x0 + lx < T.W && y0 + ly < T.H) ? g.row0 + (int64_t)ly * T.W + lx : -1;
-    return g;
-}
+};
 
-// Issues the copies of one chunk into buffer `b` (a chunk that is not entirely
-// inside the frame or not 16-byte aligned is read with plain bounded loads
-// instead; lanes without a fragment become background).
+// This lane's share of a chunk's copies.  Piece q of a chunk (0-23 dir, 24-39
+// uv, 40-47 obj) is 16 bytes of one stream, all in one tile row; lanes take
+// pieces lane and lane + 32.  A piece starts at p + m row0 bytes: m is the
+// stream's bytes per fragment, and p holds the rest, fixed for the launch.
+struct LaneCopy {
+    const char* p;
+    uint32_t m;
+
+    __device__ __forceinline__ LaneCopy(const float* dir, const float* uv, const int32_t* obj, int q, int tw_log2,
+                                        int64_t pitch) {
+        const int k = q < 24 ? 3 : q < 40 ? 2 : 1;             // values per fragment
+        const int e = 4 * (q - (q < 24 ? 0 : q < 40 ? 24 : 40));  // first value of the piece
+        const int row = (e / k) >> tw_log2;
+        const char* base = reinterpret_cast<const char*>(q < 24 ? (const void*)dir : q < 40 ? (const void*)uv : obj);
+        p = base + 4 * (k * ((int64_t)row * pitch) + (e - k * (row << tw_log2)));
+        m = 4 * k;
+    }
+    __device__ __forceinline__ const void* at(int64_t row0) const { return p + row0 * (int64_t)m; }
+};
+
+// Issues the copies of one chunk into the buffer at shared address s.  A chunk
+// that crosses the frame's edge or has unaligned rows is copied fragment by
+// fragment, each lane its own; lanes without a fragment become background.
 template <bool EXTRA, int STAGES, bool NRM>
 __device__ __forceinline__ void stage_chunk(const float* __restrict__ uv, const float* __restrict__ dir,
                                             const int32_t* __restrict__ obj, const float* __restrict__ extra,
-                                            const float* __restrict__ nrm, const ChunkGeom& g, int b,
-                                            WarpStage<EXTRA, STAGES, NRM>& S, int lane) {
+                                            const float* __restrict__ nrm, const Chunk& g, const LaneCopy& c0,
+                                            const LaneCopy& c1, unsigned s, int lane) {
+    using S = WarpStage<EXTRA, STAGES, NRM>;
     if (g.fast) {
-        // 24 pieces of dir, 16 of uv, 8 of obj: lanes 0-23 take dir, 16-31 uv,
-        // 24-31 obj.  Shared memory holds the chunk in lane order (lane = row
-        // tw + column), so piece q covers shared floats 4q..4q+3 of its stream,
-        // all in one row: row k = (first lane of the piece) >> log2(tw).
-        const int lg = g.tw_log2;
-        if (lane < 24) {
-            const int m = 4 * lane, k = (m / 3) >> lg;
-            const int64_t src = 3 * (g.row0 + (int64_t)k * g.pitch) + (m - 3 * (k << lg));
-            cp_async16(&S.dir[b][m], dir + src);
-            if (NRM) cp_async16(&S.nrm[NRM ? b : 0][NRM ? m : 0], nrm + src);
-        }
-        if (lane >= 16) {
-            const int m = 4 * (lane - 16), k = (m >> 1) >> lg;
-            cp_async16(&S.uv[b][m], uv + 2 * (g.row0 + (int64_t)k * g.pitch) + (m - 2 * (k << lg)));
-        }
-        if (lane >= 24) {
-            const int m = 4 * (lane - 24), k = m >> lg;
-            cp_async16(&S.obj[b][m], obj + (g.row0 + (int64_t)k * g.pitch) + (m - (k << lg)));
-        }
-        if (EXTRA) cp_async16(&S.extra[b][lane], extra + 4 * g.f);
-    } else {
+        cp_async<16>(s + 16 * lane, c0.at(g.row0));
+        if (lane < 16) cp_async<16>(s + 512 + 16 * lane, c1.at(g.row0));
+        if (NRM && lane < 24)  // the pieces of nrm lie as those of dir
+            cp_async<16>(s + S::kNrm + 16 * lane, reinterpret_cast<const char*>(c0.at(g.row0)) +
+                                                      (reinterpret_cast<const char*>(nrm) -
+                                                       reinterpret_cast<const char*>(dir)));
+        if (EXTRA) cp_async<16>(s + S::kExtra + 16 * lane, extra + 4 * g.f);
+    } else if (g.f >= 0) {
         const int64_t f = g.f;
-        if (f >= 0) {
-            S.uv[b][2 * lane] = uv[2 * f];
-            S.uv[b][2 * lane + 1] = uv[2 * f + 1];
-            S.dir[b][3 * lane] = dir[3 * f];
-            S.dir[b][3 * lane + 1] = dir[3 * f + 1];
-            S.dir[b][3 * lane + 2] = dir[3 * f + 2];
-            S.obj[b][lane] = obj[f];
-            if (NRM) {
-                S.nrm[NRM ? b : 0][NRM ? 3 * lane : 0] = nrm[3 * f];
-                S.nrm[NRM ? b : 0][NRM ? 3 * lane + 1 : 0] = nrm[3 * f + 1];
-                S.nrm[NRM ? b : 0][NRM ? 3 * lane + 2 : 0] = nrm[3 * f + 2];
-            }
-        } else {
-            S.uv[b][2 * lane] = S.uv[b][2 * lane + 1] = 0.f;
-            S.dir[b][3 * lane] = S.dir[b][3 * lane + 1] = S.dir[b][3 * lane + 2] = 0.f;
-            S.obj[b][lane] = -1;
-            if (NRM)
-                S.nrm[NRM ? b : 0][NRM ? 3 * lane : 0] = S.nrm[NRM ? b : 0][NRM ? 3 * lane + 1 : 0] =
-                    S.nrm[NRM ? b : 0][NRM ? 3 * lane + 2 : 0] = 0.f;
+        cp_async<8>(s + S::kUv + 8 * lane, uv + 2 * f);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            cp_async<4>(s + S::kDir + 12 * lane + 4 * k, dir + 3 * f + k);
+            if (NRM) cp_async<4>(s + S::kNrm + 12 * lane + 4 * k, nrm + 3 * f + k);
         }
-        if (EXTRA)
-            S.extra[b][lane] = f >= 0 ? reinterpret_cast<const float4*>(extra)[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+        cp_async<4>(s + S::kObj + 4 * lane, obj + f);
+        if (EXTRA) cp_async<16>(s + S::kExtra + 16 * lane, extra + 4 * f);
+    } else {
+        asm volatile("st.shared.b32 [%0], %1;" ::"r"(s + S::kObj + 4 * lane), "r"(-1) : "memory");
     }
 }
 
 template <bool EXTRA, int STAGES, bool NRM>
-__device__ __forceinline__ Frag read_frag(const WarpStage<EXTRA, STAGES, NRM>& S, int b, int lane) {
+__device__ __forceinline__ Frag read_frag(const char* S, int lane) {
+    using St = WarpStage<EXTRA, STAGES, NRM>;
     Frag r;
-    float2 q = reinterpret_cast<const float2*>(S.uv[b])[lane];
+    const float2 q = reinterpret_cast<const float2*>(S + St::kUv)[lane];
+    const float* d = reinterpret_cast<const float*>(S + St::kDir) + 3 * lane;
     r.u = q.x;
     r.v = q.y;
-    r.x = S.dir[b][3 * lane];
-    r.y = S.dir[b][3 * lane + 1];
-    r.z = S.dir[b][3 * lane + 2];
-    r.o = S.obj[b][lane];
+    r.x = d[0];
+    r.y = d[1];
+    r.z = d[2];
+    r.o = reinterpret_cast<const int*>(S + St::kObj)[lane];
     r.nx = r.ny = r.nz = 0.f;
     if (NRM) {
-        r.nx = S.nrm[NRM ? b : 0][NRM ? 3 * lane : 0];
-        r.ny = S.nrm[NRM ? b : 0][NRM ? 3 * lane + 1 : 0];
-        r.nz = S.nrm[NRM ? b : 0][NRM ? 3 * lane + 2 : 0];
+        const float* n = reinterpret_cast<const float*>(S + St::kNrm) + 3 * lane;
+        r.nx = n[0];
+        r.ny = n[1];
+        r.nz = n[2];
     }
     return r;
 }
 
-template <bool TILED>
-__device__ __forceinline__ int64_t chunk_count(const Tiling& T, int64_t F, int warps) {
-    if (!TILED) return (F + kChunk - 1) / kChunk;
-    return (int64_t)T.btx * T.bty * T.views * warps;
-}
-
 // Runs body(f, frag, extra) with all 32 lanes of the warp, one fragment per
 // lane, persistent over the grid, with the G-buffer of the next STAGES - 1
-// chunks prefetched.  Lanes without a fragment get a background fragment and
-// f = -1: the body must not store for them.  WARPS = warps per block; the
-// block's shared memory holds WARPS stages.
+// chunks prefetched.  Lanes without a fragment get a background fragment
+// (object id -1, other inputs arbitrary) and f = -1: the body must not store
+// for them.  WARPS = warps per block; the block's shared memory holds WARPS
+// stages.  Bound of the shading kernels: issue, so what a chunk costs beside its
+// lookups counts: walking and copying it took about 120 of the forward's 360
+// instructions with the tile found by division and each stream's addresses
+// formed per chunk, WALK_INSTR as it is now (1080p forward, FP16 quadrilinear).
 template <int WARPS, bool EXTRA, bool TILED, int STAGES, bool NRM = false, typename Body>
 __device__ __forceinline__ void for_each_fragment(const float* __restrict__ uv, const float* __restrict__ dir,
                                                   const int32_t* __restrict__ obj, const float* __restrict__ extra,
                                                   int64_t F, const Tiling& T, WarpStage<EXTRA, STAGES, NRM>* stages,
                                                   Body body, const float* __restrict__ nrm = nullptr) {
-    constexpr int kStages = STAGES;
+    using St = WarpStage<EXTRA, STAGES, NRM>;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    WarpStage<EXTRA, STAGES, NRM>& S = stages[w];
-    const int64_t nchunks = chunk_count<TILED>(T, F, WARPS);
-    const int64_t step = (int64_t)gridDim.x * WARPS;
-    int64_t c = (int64_t)blockIdx.x * WARPS + w;
-    // fk[k]: this lane's fragment of chunk c + k * step, staged in buffer (b + k) % kStages
-    int64_t fk[kStages];
+    const char* S = stages[w].b[0];
+    const unsigned s0 = (unsigned)__cvta_generic_to_shared(S);
+    ChunkWalk<WARPS, TILED> walk(T, F, lane, w);
+    const int lg = TILED ? T.tw_log2 : 5;
+    const LaneCopy c0(dir, uv, obj, lane, lg, TILED ? T.W : 0), c1(dir, uv, obj, lane + 32, lg, TILED ? T.W : 0);
+    // fk[k]: this lane's fragment of the k-th chunk from the current one, staged in buffer (b + k) % STAGES
+    int64_t fk[STAGES];
 #pragma unroll
-    for (int k = 0; k < kStages - 1; ++k) {
-        const ChunkGeom g = chunk_geom<WARPS, TILED>(T, F, c + k * step, lane);
-        if (c + k * step < nchunks) stage_chunk<EXTRA, STAGES, NRM>(uv, dir, obj, extra, nrm, g, k, S, lane);
+    for (int k = 0; k < STAGES - 1; ++k) {
+        const Chunk g = walk.next(T, F, lane);
+        if (k < walk.count) stage_chunk<EXTRA, STAGES, NRM>(uv, dir, obj, extra, nrm, g, c0, c1, s0 + k * St::kBytes, lane);
         cp_async_commit();
         fk[k] = g.f;
     }
     int b = 0;
-    for (; c < nchunks; c += step) {
-        const int64_t ahead = c + (kStages - 1) * step;
-        const int bl = b + kStages - 1 >= kStages ? b - 1 : b + kStages - 1;  // (b + kStages - 1) % kStages
-        const ChunkGeom g = chunk_geom<WARPS, TILED>(T, F, ahead, lane);
-        if (ahead < nchunks) stage_chunk<EXTRA, STAGES, NRM>(uv, dir, obj, extra, nrm, g, bl, S, lane);
+    for (int64_t left = walk.count; left > 0; --left) {
+        const Chunk g = walk.next(T, F, lane);
+        const int bl = b + STAGES - 1 >= STAGES ? b - 1 : b + STAGES - 1;  // (b + STAGES - 1) % STAGES
+        if (left > STAGES - 1)
+            stage_chunk<EXTRA, STAGES, NRM>(uv, dir, obj, extra, nrm, g, c0, c1, s0 + bl * St::kBytes, lane);
         cp_async_commit();
-        fk[kStages - 1] = g.f;
-        cp_async_wait<kStages - 1>();  // chunk c has landed (newer groups may still be in flight)
+        fk[STAGES - 1] = g.f;
+        cp_async_wait<STAGES - 1>();  // the current chunk has landed (newer groups may still be in flight)
         __syncwarp();
-        const Frag q = read_frag<EXTRA, STAGES, NRM>(S, b, lane);
+        const Frag q = read_frag<EXTRA, STAGES, NRM>(S + b * St::kBytes, lane);
         float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (EXTRA) e = S.extra[EXTRA ? b : 0][EXTRA ? lane : 0];
+        if (EXTRA) e = reinterpret_cast<const float4*>(S + b * St::kBytes + St::kExtra)[lane];
         __syncwarp();  // every lane has read buffer b before it is refilled
         body(fk[0], q, e);
 #pragma unroll
-        for (int k = 0; k < kStages - 1; ++k) fk[k] = fk[k + 1];
-        b = b + 1 == kStages ? 0 : b + 1;
+        for (int k = 0; k < STAGES - 1; ++k) fk[k] = fk[k + 1];
+        b = b + 1 == STAGES ? 0 : b + 1;
     }
     cp_async_wait<0>();
 }
