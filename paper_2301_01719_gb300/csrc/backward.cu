@@ -54,7 +54,7 @@ static cudaError_t launch_backward_t(const TexDesc* table, int n_obj, const floa
                                      const int32_t* obj, int64_t F, const Tiling& T, const float* dL_dout,
                                      const GradTable& grads, bool any_grad, float* dL_duv, float* dL_ddir,
                                      bool accumulate, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(backward_kernel<FILTER, TILED, DET, SPEC>, kBackThreads,
+    const unsigned grid = persistent_grid<backward_kernel<FILTER, TILED, DET, SPEC>>(kBackThreads,
                                           chunk_count_host(T, F, kBackWarps));
     backward_kernel<FILTER, TILED, DET, SPEC><<<grid, kBackThreads, 0, stream>>>(
         table, n_obj, uv, dir, obj, F, T, dL_dout, grads, any_grad, dL_duv, dL_ddir, accumulate, status);
@@ -180,7 +180,7 @@ static cudaError_t launch_world_backward_t(const TexDesc* table, int n_obj, cons
                                            const float* dL_dout, const GradTable& grads, bool any_grad, float* dL_duv,
                                            float* dL_ddir, float* dL_dnrm, bool accumulate, unsigned* status,
                                            cudaStream_t stream) {
-    const unsigned grid = persistent_grid(world_backward_kernel<FILTER, DET, TILED>, kBackThreads,
+    const unsigned grid = persistent_grid<world_backward_kernel<FILTER, DET, TILED>>(kBackThreads,
                                           chunk_count_host(T, F, kBackWarps));
     world_backward_kernel<FILTER, DET, TILED><<<grid, kBackThreads, 0, stream>>>(
         table, n_obj, uv, dir, nrm, obj, F, T, dL_dout, grads, any_grad, dL_duv, dL_ddir, dL_dnrm, accumulate,

@@ -141,7 +141,7 @@ static cudaError_t launch_fused_t(const TexDesc* table, int n_obj, const float* 
                                   const int32_t* obj, int64_t F, const Tiling& T, const float* target, float scale,
                                   float* out, double* sums, const GradTable& grads, bool any_grad, float* dL_duv,
                                   float* dL_ddir, bool accumulate, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(fused_l2_kernel<FILTER, DET, SPEC>, kBackThreads,
+    const unsigned grid = persistent_grid<fused_l2_kernel<FILTER, DET, SPEC>>(kBackThreads,
                                           chunk_count_host(T, F, kBackWarps));
     fused_l2_kernel<FILTER, DET, SPEC><<<grid, kBackThreads, 0, stream>>>(
         table, n_obj, uv, dir, obj, F, T, target, scale, out, sums, grads, any_grad, dL_duv, dL_ddir, accumulate,

@@ -470,10 +470,11 @@ __device__ __forceinline__ Frag read_frag(const char* S, int lane) {
 // chunks prefetched.  Lanes without a fragment get a background fragment
 // (object id -1, other inputs arbitrary) and f = -1: the body must not store
 // for them.  WARPS = warps per block; the block's shared memory holds WARPS
-// stages.  Bound of the shading kernels: issue, so what a chunk costs beside its
-// lookups counts: walking and copying it took about 120 of the forward's 360
-// instructions with the tile found by division and each stream's addresses
-// formed per chunk, WALK_INSTR as it is now (1080p forward, FP16 quadrilinear).
+// stages.  Bound of the shading kernels: issue and latency, so what a chunk costs
+// beside its lookups counts: with the tile found by division and each stream's
+// addresses formed per chunk the 1080p FP16 quadrilinear forward took 360
+// instructions per chunk, with the walk and the lane's pointers 316 (20 poses:
+// 0.586 -> 0.498 ms).
 template <int WARPS, bool EXTRA, bool TILED, int STAGES, bool NRM = false, typename Body>
 __device__ __forceinline__ void for_each_fragment(const float* __restrict__ uv, const float* __restrict__ dir,
                                                   const int32_t* __restrict__ obj, const float* __restrict__ extra,

@@ -109,7 +109,7 @@ template <int FILTER, bool TILED>
 static cudaError_t launch_world_shade_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                         const float* nrm, const int32_t* obj, int64_t F, const Tiling& T, float* out,
                                         int32_t* idx, float* coord, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(world_shade_kernel<FILTER, TILED>, kShadeThreads,
+    const unsigned grid = persistent_grid<world_shade_kernel<FILTER, TILED>>(kShadeThreads,
                                           chunk_count_host(T, F, kShadeWarps));
     world_shade_kernel<FILTER, TILED><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dir, nrm, obj, F, T,
                                                                           out, idx, coord, status);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kShadeThreads, 8) multi_bits_kernel(const TexD
 template <int FILTER, int KIND>
 static void launch_multi_bits(const TexDesc* table, int n_obj, const float* uv, const float* dirs, int S,
                               const int32_t* obj, int64_t F, float* out, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(multi_bits_kernel<FILTER, KIND>, kShadeThreads, (F + 32 / S - 1) / (32 / S));
+    const unsigned grid = persistent_grid<multi_bits_kernel<FILTER, KIND>>(kShadeThreads, (F + 32 / S - 1) / (32 / S));
     multi_bits_kernel<FILTER, KIND><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out, status);
 }
 
@@ -318,11 +318,11 @@ static void launch_multi_t(const TexDesc* table, int n_obj, const float* uv, con
     } else if (S <= 32 && bits == kBitsLarge) {
         launch_multi_bits<FILTER, kBitsLarge>(table, n_obj, uv, dirs, S, obj, F, out, status, stream);
     } else if (S <= 32 && (S & (S - 1)) == 0) {
-        const unsigned grid = persistent_grid(multi_shade_lanes_kernel<FILTER>, kShadeThreads, (F * S + 31) / 32);
+        const unsigned grid = persistent_grid<multi_shade_lanes_kernel<FILTER>>(kShadeThreads, (F * S + 31) / 32);
         multi_shade_lanes_kernel<FILTER><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out,
                                                                               status);
     } else {
-        const unsigned grid = persistent_grid(multi_shade_kernel<FILTER>, kShadeThreads,
+        const unsigned grid = persistent_grid<multi_shade_kernel<FILTER>>(kShadeThreads,
                                               (F + kShadeThreads - 1) / kShadeThreads);
         multi_shade_kernel<FILTER><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out,
                                                                         status);
@@ -349,7 +349,7 @@ template <int FILTER, bool TILED, int SPEC>
 static cudaError_t launch_shade_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                   const int32_t* obj, int64_t F, const Tiling& T, float* out, unsigned* status,
                                   cudaStream_t stream) {
-    const unsigned grid = persistent_grid(shade_kernel<FILTER, TILED, SPEC>, kShadeThreads,
+    const unsigned grid = persistent_grid<shade_kernel<FILTER, TILED, SPEC>>(kShadeThreads,
                                           chunk_count_host(T, F, kShadeWarps));
     shade_kernel<FILTER, TILED, SPEC><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dir, obj, F, T, out,
                                                                           status);
@@ -399,7 +399,7 @@ template <int FILTER, bool TILED>
 static cudaError_t launch_locate_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                    const int32_t* obj, int64_t F, const Tiling& T, int32_t* idx, float* coord,
                                    unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(locate_kernel<FILTER, TILED>, kShadeThreads,
+    const unsigned grid = persistent_grid<locate_kernel<FILTER, TILED>>(kShadeThreads,
                                           chunk_count_host(T, F, kShadeWarps));
     locate_kernel<FILTER, TILED><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dir, obj, F, T, idx, coord,
                                                                      status);

@@ -354,7 +354,7 @@ template <int FILTER>
 static cudaError_t launch_footprint_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                       const int32_t* obj, int64_t F, uint32_t* bitmap, const int64_t* word_offset,
                                       unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid(footprint_kernel<FILTER>, kThreads, (F + kChunk - 1) / kChunk);
+    const unsigned grid = persistent_grid<footprint_kernel<FILTER>>(kThreads, (F + kChunk - 1) / kChunk);
     footprint_kernel<FILTER><<<grid, kThreads, 0, stream>>>(table, n_obj, uv, dir, obj, F, bitmap, word_offset,
                                                             status);
     return cudaGetLastError();
