@@ -28,7 +28,7 @@ struct rt_ctx {
     int tile[2][3][4];                   // per pass (forward, backward) and filter: tw, th, bx, by of the batched kernels
     long long* det[RT_MAX_OBJECTS];      // fixed-point gradient sums of the deterministic mode
     uint32_t* index[RT_MAX_OBJECTS];     // palette index maps the library copied
-    int spec = -1;                       // the format shared by all objects (dense PLANES, clamp), else -1
+    int spec = -1;                       // the format (+ kSpecPalette) shared by all objects in clamp mode, else -1
     int bits = rt::kBitsNone;            // how the bits are indexed if all objects are bit textures in clamp mode
     uint32_t wait_limit = 0;             // polls of a bounded device wait before it gives up (0: the default)
 };
@@ -94,16 +94,19 @@ rt_status check_gbuffer(const float* uv, const float* dir, const int32_t* obj, i
     return RT_OK;
 }
 
-// The single-format specialisation the tiled kernels may use for this table.
+// The single-format specialisation the tiled kernels may use for this table:
+// all objects of one format in clamp mode, all dense or all palettes.
 int table_spec(const rt_ctx* ctx) {
     int spec = -2;
     for (int o = 0; o < ctx->n_obj; ++o) {
         const TexDesc& d = ctx->table[o];
         if (!d.live) continue;
-        if (d.layout != RT_LAYOUT_QUADS || d.wrap || d.fmt == RT_BIT1) return -1;
+        const bool palette = d.layout == rt::kLayoutPalette;
+        if ((d.layout != RT_LAYOUT_QUADS && !palette) || d.wrap || d.fmt == RT_BIT1) return -1;
+        const int s = palette ? d.fmt + rt::kSpecPalette : d.fmt;
         if (spec == -2)
-            spec = d.fmt;
-        else if (spec != d.fmt)
+            spec = s;
+        else if (spec != s)
             return -1;
     }
     return spec < 0 ? -1 : spec;
@@ -638,8 +641,8 @@ static rt_status shade_backward_impl(rt_ctx* ctx, const float* uv, const float* 
     }
     if (e == cudaSuccess && F > 0) {
         if (nrm)
-            e = rt::launch_world_backward(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter, T, dL_dout, grads,
-                                          any, dL_duv, dL_ddir, dL_dnrm, accumulate, deterministic, ctx->d_status, s);
+            e = rt::launch_world_backward(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter, T, ctx->spec, dL_dout,
+                                          grads, any, dL_duv, dL_ddir, dL_dnrm, accumulate, deterministic, ctx->d_status, s);
         else if (fused)
             e = rt::launch_fused_l2(ctx->d_table, ctx->n_obj, uv, dir, obj, F, filter, T, ctx->spec, fused->target,
                                     fused->scale, fused->out, fused->sums, grads, any, dL_duv, dL_ddir, accumulate,
@@ -771,7 +774,7 @@ rt_status rt_shade_world(rt_ctx* ctx, const float* uv, const float* dir, const f
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
     return cuda_status(rt::launch_world_shade(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter,
-                                              rt::flat_tiling(), out, nullptr, nullptr, ctx->d_status,
+                                              rt::flat_tiling(), -1, out, nullptr, nullptr, ctx->d_status,
                                               (cudaStream_t)stream));
 }
 
@@ -785,7 +788,7 @@ rt_status rt_locate_world(rt_ctx* ctx, const float* uv, const float* dir, const 
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
     return cuda_status(rt::launch_world_shade(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter,
-                                              rt::flat_tiling(), nullptr, idx, coord, ctx->d_status,
+                                              rt::flat_tiling(), -1, nullptr, idx, coord, ctx->d_status,
                                               (cudaStream_t)stream));
 }
 
@@ -857,8 +860,8 @@ rt_status rt_shade_world_batched(rt_ctx* ctx, const float* uv, const float* dir,
     if (!frames_tiling(ctx, kForward, views, height, width, filter, &T)) return RT_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
-    return cuda_status(rt::launch_world_shade(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter, T, out, nullptr,
-                                              nullptr, ctx->d_status, (cudaStream_t)stream));
+    return cuda_status(rt::launch_world_shade(ctx->d_table, ctx->n_obj, uv, dir, nrm, obj, F, filter, T, ctx->spec, out,
+                                              nullptr, nullptr, ctx->d_status, (cudaStream_t)stream));
 }
 
 rt_status rt_shade_world_batched_backward(rt_ctx* ctx, const float* uv, const float* dir, const float* nrm,

@@ -115,8 +115,8 @@ cudaError_t launch_backward(const TexDesc* table, int n_obj, const float* uv, co
 // the tangent-space backward with the normal as a fourth staged stream, over
 // the flat fragment stream or, TILED, over screen tiles of a batch of frames.
 // dL/dI = dL/dN, since A depends on h = I + N only.
-template <int FILTER, bool DET, bool TILED>
-__global__ void __launch_bounds__(kBackThreads) world_backward_kernel(
+template <int FILTER, bool DET, bool TILED, int SPEC>
+__global__ void __launch_bounds__(kBackThreads, SPEC >= 0 ? 6 : 1) world_backward_kernel(
     const TexDesc* __restrict__ table, int n_obj, const float* __restrict__ uv, const float* __restrict__ dir,
     const float* __restrict__ nrm, const int32_t* __restrict__ obj, int64_t F, Tiling tiling,
     const float* __restrict__ dL_dout,
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kBackThreads) world_backward_kernel(
         const bool valid = fragment_valid(table, n_obj, q.o, q.u, q.v, I.x, I.y, I.z, status, d) &&
                            normal_valid(N, status);
         if (valid) {
-            L = locate_world<FILTER>(d, q.u, q.v, I, N);
+            L = locate_world<FILTER, (SPEC < 0)>(d, q.u, q.v, I, N);
             if (any_grad) grad = grads.p[q.o];
         }
         if (DET) {
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kBackThreads) world_backward_kernel(
             grad = nullptr;
         }
         if (valid && (!DET || coord_grads)) {
-            const CoordGrad cg = backward_any<FILTER>(d, L, go, grad, coord_grads);
+            const CoordGrad cg = backward_spec<FILTER, SPEC>(d, L, go, grad, coord_grads);
             if (FILTER == RT_QUADRILINEAR) guv = uv_grad(d, q.u, q.v, cg.gu, cg.gv);
             if (FILTER != RT_NEAREST && (dL_ddir || dL_dnrm)) {
                 const float gBx = (L.B.x > -d.hi && L.B.x < d.hi) ? cg.gs * d.half_n : 0.f;
@@ -174,28 +174,28 @@ __global__ void __launch_bounds__(kBackThreads) world_backward_kernel(
     }, nrm);
 }
 
-template <int FILTER, bool DET, bool TILED>
+template <int FILTER, bool DET, bool TILED, int SPEC>
 static cudaError_t launch_world_backward_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                            const float* nrm, const int32_t* obj, int64_t F, const Tiling& T,
                                            const float* dL_dout, const GradTable& grads, bool any_grad, float* dL_duv,
                                            float* dL_ddir, float* dL_dnrm, bool accumulate, unsigned* status,
                                            cudaStream_t stream) {
-    const unsigned grid = persistent_grid<world_backward_kernel<FILTER, DET, TILED>>(kBackThreads,
+    const unsigned grid = persistent_grid<world_backward_kernel<FILTER, DET, TILED, SPEC>>(kBackThreads,
                                           chunk_count_host(T, F, kBackWarps));
-    world_backward_kernel<FILTER, DET, TILED><<<grid, kBackThreads, 0, stream>>>(
+    world_backward_kernel<FILTER, DET, TILED, SPEC><<<grid, kBackThreads, 0, stream>>>(
         table, n_obj, uv, dir, nrm, obj, F, T, dL_dout, grads, any_grad, dL_duv, dL_ddir, dL_dnrm, accumulate,
         status);
     return cudaGetLastError();
 }
 
-template <bool DET, bool TILED>
+template <bool DET, bool TILED, int SPEC>
 static cudaError_t launch_world_backward_d(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                            const float* nrm, const int32_t* obj, int64_t F, int filter,
                                            const Tiling& T, const float* dL_dout, const GradTable& grads,
                                            bool any_grad, float* dL_duv, float* dL_ddir, float* dL_dnrm,
                                            bool accumulate, unsigned* status, cudaStream_t stream) {
 #define RT_WBWD(FILT)                                                                                              \
-    launch_world_backward_t<FILT, DET, TILED>(table, n_obj, uv, dir, nrm, obj, F, T, dL_dout, grads, any_grad,      \
+    launch_world_backward_t<FILT, DET, TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, T, dL_dout, grads, any_grad,      \
                                               dL_duv, dL_ddir, dL_dnrm, accumulate, status, stream)
     switch (filter) {
         case RT_NEAREST:
@@ -210,14 +210,26 @@ static cudaError_t launch_world_backward_d(const TexDesc* table, int n_obj, cons
 
 cudaError_t launch_world_backward(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                   const float* nrm, const int32_t* obj, int64_t F, int filter, const Tiling& T,
-                                  const float* dL_dout, const GradTable& grads, bool any_grad, float* dL_duv,
-                                  float* dL_ddir, float* dL_dnrm, bool accumulate, bool deterministic,
+                                  int spec, const float* dL_dout, const GradTable& grads, bool any_grad,
+                                  float* dL_duv, float* dL_ddir, float* dL_dnrm, bool accumulate, bool deterministic,
                                   unsigned* status, cudaStream_t stream) {
-#define RT_WBWD_D(DET, TILED)                                                                                      \
-    launch_world_backward_d<DET, TILED>(table, n_obj, uv, dir, nrm, obj, F, filter, T, dL_dout, grads, any_grad,    \
-                                        dL_duv, dL_ddir, dL_dnrm, accumulate, status, stream)
-    if (T.W > 0) return deterministic ? RT_WBWD_D(true, true) : RT_WBWD_D(false, true);
-    return deterministic ? RT_WBWD_D(true, false) : RT_WBWD_D(false, false);
+#define RT_WBWD_D(DET, TILED, SPEC)                                                                               \
+    launch_world_backward_d<DET, TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, filter, T, dL_dout, grads,       \
+                                              any_grad, dL_duv, dL_ddir, dL_dnrm, accumulate, status, stream)
+    if (T.W <= 0) return deterministic ? RT_WBWD_D(true, false, -1) : RT_WBWD_D(false, false, -1);
+    if (deterministic) return RT_WBWD_D(true, true, -1);
+    switch (spec) {
+        case RT_F16:
+            return RT_WBWD_D(false, true, RT_F16);
+        case RT_BF16:
+            return RT_WBWD_D(false, true, RT_BF16);
+        case RT_F32:
+            return RT_WBWD_D(false, true, RT_F32);
+        case RT_E4M3_BUCKET_SCALE:
+            return RT_WBWD_D(false, true, RT_E4M3_BUCKET_SCALE);
+        default:
+            return RT_WBWD_D(false, true, -1);
+    }
 #undef RT_WBWD_D
 }
 

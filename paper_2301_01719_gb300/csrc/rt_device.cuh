@@ -241,9 +241,9 @@ __device__ __forceinline__ Lookup<FILTER> locate(const TexDesc& d, float u, floa
 }
 
 // World-space lookup: A from the first two entries of Eq. 1a, h = I + N.
-template <int FILTER>
+template <int FILTER, bool WRAP = true>
 __device__ __forceinline__ Lookup<FILTER> locate_world(const TexDesc& d, float u, float v, float3 I, float3 N) {
-    return locate_from_square<FILTER>(d, u, v, square_from_half(I.x + N.x, I.y + N.y, I.z + N.z));
+    return locate_from_square<FILTER, WRAP>(d, u, v, square_from_half(I.x + N.x, I.y + N.y, I.z + N.z));
 }
 
 // ---------------------------------------------------------------------------

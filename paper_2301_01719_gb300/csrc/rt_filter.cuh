@@ -218,14 +218,17 @@ __device__ __forceinline__ float4 filter_any(const TexDesc& d, const Lookup<FILT
 
 // SPEC: -1 = any objects (format, layout, palette and repeat mode dispatched
 // per fragment); a format = every object of the table is a dense QUADS
-// texture of that format in clamp mode, so the fragment code is one path
-// (the host picks the instantiation from the table).
+// texture of that format in clamp mode, a format + kSpecPalette = a palette of
+// that format in clamp mode, so the fragment code is one path (the host picks
+// the instantiation from the table).
+constexpr int kSpecPalette = 16;
+
 template <int FILTER, int SPEC>
 __device__ __forceinline__ float4 filter_spec(const TexDesc& d, const Lookup<FILTER>& L) {
     if constexpr (SPEC < 0)
         return filter_any<FILTER>(d, L);
     else
-        return filter_taps<FILTER, SPEC, RT_LAYOUT_QUADS>(d, L);
+        return filter_taps<FILTER, SPEC % kSpecPalette, SPEC < kSpecPalette ? RT_LAYOUT_QUADS : kLayoutPalette>(d, L);
 }
 
 // G-buffer staging.  Kernels that walk fragments are persistent: each warp

@@ -63,7 +63,8 @@ struct GradTable {
 };
 
 // spec: the storage format shared by every object of the table (dense QUADS,
-// clamp mode), or -1; selects a single-format instantiation of the tiled kernels.
+// clamp mode), that + kSpecPalette if all are palettes, or -1; selects a
+// single-format instantiation of the tiled kernels where there is one.
 cudaError_t launch_shade(const TexDesc* table, int n_obj, const float* uv, const float* dir, const int32_t* obj,
                          int64_t F, int filter, const Tiling& T, int spec, float* out, unsigned* status,
                          cudaStream_t stream);
@@ -93,12 +94,12 @@ cudaError_t launch_multi_shade(const TexDesc* table, int n_obj, const float* uv,
                                cudaStream_t stream);
 // World-space kernels: T is flat_tiling() for the flat stream, or a screen tiling.
 cudaError_t launch_world_shade(const TexDesc* table, int n_obj, const float* uv, const float* dir, const float* nrm,
-                               const int32_t* obj, int64_t F, int filter, const Tiling& T, float* out, int32_t* idx,
-                               float* coord, unsigned* status, cudaStream_t stream);
+                               const int32_t* obj, int64_t F, int filter, const Tiling& T, int spec, float* out,
+                               int32_t* idx, float* coord, unsigned* status, cudaStream_t stream);
 cudaError_t launch_world_backward(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                   const float* nrm, const int32_t* obj, int64_t F, int filter, const Tiling& T,
-                                  const float* dL_dout, const GradTable& grads, bool any_grad, float* dL_duv,
-                                  float* dL_ddir, float* dL_dnrm, bool accumulate, bool deterministic,
+                                  int spec, const float* dL_dout, const GradTable& grads, bool any_grad,
+                                  float* dL_duv, float* dL_ddir, float* dL_dnrm, bool accumulate, bool deterministic,
                                   unsigned* status, cudaStream_t stream);
 int64_t kmeans_tc_scratch_bytes(int W, int H, int n, int K);
 // converted: the scratch holds the bucket vectors and their norms already.

@@ -17,22 +17,22 @@ namespace rt {
 constexpr int kShadeThreads = 128;
 constexpr int kShadeWarps = kShadeThreads / 32;
 
-// The screen-tiled forward keeps three G-buffer chunks per warp (two in
-// flight) and is held to 64 registers, 8 blocks (32 warps) per SM: measured 4%
-// faster than two chunks at 72 registers.  The flat stream keeps two chunks
-// (it would spill at 64 registers).
-template <bool TILED>
-constexpr int shade_stages() { return TILED ? 3 : 2; }
+// The screen-tiled and the single-format forward keep three G-buffer chunks per
+// warp (two in flight) and are held to 64 registers, 8 blocks (32 warps) per SM:
+// measured 4% faster than two chunks at 72 registers.  The dispatching kernel of
+// the flat stream keeps two chunks (it would spill at 64 registers).
+template <bool TILED, int SPEC>
+constexpr int shade_stages() { return TILED || SPEC >= 0 ? 3 : 2; }
 
 template <int FILTER, bool TILED, int SPEC>
-__global__ void __launch_bounds__(kShadeThreads, TILED ? 8 : 1) shade_kernel(const TexDesc* __restrict__ table, int n_obj,
+__global__ void __launch_bounds__(kShadeThreads, TILED || SPEC >= 0 ? 8 : 1) shade_kernel(const TexDesc* __restrict__ table, int n_obj,
                                                               const float* __restrict__ uv,
                                                               const float* __restrict__ dir,
                                                               const int32_t* __restrict__ obj, int64_t F,
                                                               Tiling tiling, float* __restrict__ out,
                                                               unsigned* status) {
-    __shared__ WarpStage<false, shade_stages<TILED>()> stages[kShadeWarps];
-    for_each_fragment<kShadeWarps, false, TILED, shade_stages<TILED>()>(uv, dir, obj, nullptr, F, tiling, stages,
+    __shared__ WarpStage<false, shade_stages<TILED, SPEC>()> stages[kShadeWarps];
+    for_each_fragment<kShadeWarps, false, TILED, shade_stages<TILED, SPEC>()>(uv, dir, obj, nullptr, F, tiling, stages,
                                                                [&](int64_t f, const Frag& q, float4) {
         float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
         TexDesc d;
@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(kShadeThreads) locate_kernel(const TexDesc* __
 // streamer of the tangent-space kernels with a fourth staged stream, the
 // normal, over the flat fragment stream or, TILED, over screen tiles of a batch
 // of frames.
-template <int FILTER, bool TILED>
-__global__ void __launch_bounds__(kShadeThreads) world_shade_kernel(const TexDesc* __restrict__ table, int n_obj,
+template <int FILTER, bool TILED, int SPEC>
+__global__ void __launch_bounds__(kShadeThreads, SPEC >= 0 ? 8 : 1) world_shade_kernel(const TexDesc* __restrict__ table, int n_obj,
                                                                     const float* __restrict__ uv,
                                                                     const float* __restrict__ dir,
                                                                     const float* __restrict__ nrm,
@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(kShadeThreads) world_shade_kernel(const TexDes
         TexDesc d;
         const float3 N = make_float3(q.nx, q.ny, q.nz);
         if (fragment_valid(table, n_obj, q.o, q.u, q.v, q.x, q.y, q.z, status, d) && normal_valid(N, status)) {
-            const Lookup<FILTER> L = locate_world<FILTER>(d, q.u, q.v, make_float3(q.x, q.y, q.z), N);
-            if (out) res = filter_any<FILTER>(d, L);
+            const Lookup<FILTER> L = locate_world<FILTER, (SPEC < 0)>(d, q.u, q.v, make_float3(q.x, q.y, q.z), N);
+            if (out) res = filter_spec<FILTER, SPEC>(d, L);
             Ix = make_int4(L.u.fl, L.v.fl, L.s.fl, L.t.fl);
             C = make_float4(L.u.c, L.v.c, L.s.c, L.t.c);
         }
@@ -105,43 +105,58 @@ __global__ void __launch_bounds__(kShadeThreads) world_shade_kernel(const TexDes
     }, nrm);
 }
 
-template <int FILTER, bool TILED>
+template <int FILTER, bool TILED, int SPEC>
 static cudaError_t launch_world_shade_t(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                         const float* nrm, const int32_t* obj, int64_t F, const Tiling& T, float* out,
                                         int32_t* idx, float* coord, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid<world_shade_kernel<FILTER, TILED>>(kShadeThreads,
+    const unsigned grid = persistent_grid<world_shade_kernel<FILTER, TILED, SPEC>>(kShadeThreads,
                                           chunk_count_host(T, F, kShadeWarps));
-    world_shade_kernel<FILTER, TILED><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dir, nrm, obj, F, T,
+    world_shade_kernel<FILTER, TILED, SPEC><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dir, nrm, obj, F, T,
                                                                           out, idx, coord, status);
     return cudaGetLastError();
 }
 
-template <bool TILED>
+template <bool TILED, int SPEC>
 static cudaError_t launch_world_shade_f(const TexDesc* table, int n_obj, const float* uv, const float* dir,
                                         const float* nrm, const int32_t* obj, int64_t F, int filter, const Tiling& T,
                                         float* out, int32_t* idx, float* coord, unsigned* status,
                                         cudaStream_t stream) {
     switch (filter) {
         case RT_NEAREST:
-            return launch_world_shade_t<RT_NEAREST, TILED>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx, coord,
+            return launch_world_shade_t<RT_NEAREST, TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx, coord,
                                                            status, stream);
         case RT_ANGULAR_BILINEAR:
-            return launch_world_shade_t<RT_ANGULAR_BILINEAR, TILED>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx,
+            return launch_world_shade_t<RT_ANGULAR_BILINEAR, TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx,
                                                                     coord, status, stream);
         default:
-            return launch_world_shade_t<RT_QUADRILINEAR, TILED>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx,
+            return launch_world_shade_t<RT_QUADRILINEAR, TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, T, out, idx,
                                                                 coord, status, stream);
     }
 }
 
+// Single-format instantiations of the screen-tiled path as for the tangent-space
+// lookup: 64 registers and 8 blocks per SM instead of 112 and 4.  Forward and
+// coordinate gradients of 12 poses of 1080p, FP16: 0.918 ms dispatching, 0.824 ms
+// with these and the backward's (80 registers, 6 blocks, instead of 136 and 3).
 cudaError_t launch_world_shade(const TexDesc* table, int n_obj, const float* uv, const float* dir, const float* nrm,
-                               const int32_t* obj, int64_t F, int filter, const Tiling& T, float* out, int32_t* idx,
-                               float* coord, unsigned* status, cudaStream_t stream) {
-    if (T.W > 0)
-        return launch_world_shade_f<true>(table, n_obj, uv, dir, nrm, obj, F, filter, T, out, idx, coord, status,
-                                          stream);
-    return launch_world_shade_f<false>(table, n_obj, uv, dir, nrm, obj, F, filter, T, out, idx, coord, status,
-                                       stream);
+                               const int32_t* obj, int64_t F, int filter, const Tiling& T, int spec, float* out,
+                               int32_t* idx, float* coord, unsigned* status, cudaStream_t stream) {
+#define RT_WSHADE(TILED, SPEC)                                                                                    \
+    launch_world_shade_f<TILED, SPEC>(table, n_obj, uv, dir, nrm, obj, F, filter, T, out, idx, coord, status, stream)
+    if (T.W <= 0) return RT_WSHADE(false, -1);
+    switch (spec) {
+        case RT_F16:
+            return RT_WSHADE(true, RT_F16);
+        case RT_BF16:
+            return RT_WSHADE(true, RT_BF16);
+        case RT_F32:
+            return RT_WSHADE(true, RT_F32);
+        case RT_E4M3_BUCKET_SCALE:
+            return RT_WSHADE(true, RT_E4M3_BUCKET_SCALE);
+        default:
+            return RT_WSHADE(true, -1);
+    }
+#undef RT_WSHADE
 }
 
 // S lookups per fragment, averaged (area lights over a shadow texture, Section
@@ -372,27 +387,37 @@ static cudaError_t launch_shade_f(const TexDesc* table, int n_obj, const float* 
     }
 }
 
-// The screen-tiled path has a single-format instantiation per storage format
-// (spec = that format); everything else runs the dispatching kernels.
+// A single-format instantiation per storage format, dense and palette (spec);
+// contexts of several formats, with repeating or with borrowed objects of another
+// layout run the dispatching kernels.  20 poses of 1080p, E4M3 palettes of 1024
+// buckets: 0.591 ms dispatching (64 registers, spilling), 0.547 ms here (56).
+template <bool TILED>
+static cudaError_t launch_shade_s(const TexDesc* table, int n_obj, const float* uv, const float* dir,
+                                  const int32_t* obj, int64_t F, int filter, const Tiling& T, int spec, float* out,
+                                  unsigned* status, cudaStream_t stream) {
+#define RT_SHADE(SPEC)  \
+    case SPEC:          \
+        return launch_shade_f<TILED, SPEC>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream)
+    switch (spec) {
+        RT_SHADE(RT_F16);
+        RT_SHADE(RT_BF16);
+        RT_SHADE(RT_F32);
+        RT_SHADE(RT_E4M3_BUCKET_SCALE);
+        RT_SHADE(RT_F16 + kSpecPalette);
+        RT_SHADE(RT_BF16 + kSpecPalette);
+        RT_SHADE(RT_F32 + kSpecPalette);
+        RT_SHADE(RT_E4M3_BUCKET_SCALE + kSpecPalette);
+        default:
+            return launch_shade_f<TILED, -1>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
+    }
+#undef RT_SHADE
+}
+
 cudaError_t launch_shade(const TexDesc* table, int n_obj, const float* uv, const float* dir, const int32_t* obj,
                          int64_t F, int filter, const Tiling& T, int spec, float* out, unsigned* status,
                          cudaStream_t stream) {
-    if (T.W > 0) {
-        switch (spec) {
-            case RT_F16:
-                return launch_shade_f<true, RT_F16>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
-            case RT_BF16:
-                return launch_shade_f<true, RT_BF16>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
-            case RT_F32:
-                return launch_shade_f<true, RT_F32>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
-            case RT_E4M3_BUCKET_SCALE:
-                return launch_shade_f<true, RT_E4M3_BUCKET_SCALE>(table, n_obj, uv, dir, obj, F, filter, T, out,
-                                                                  status, stream);
-            default:
-                return launch_shade_f<true, -1>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
-        }
-    }
-    return launch_shade_f<false, -1>(table, n_obj, uv, dir, obj, F, filter, T, out, status, stream);
+    if (T.W > 0) return launch_shade_s<true>(table, n_obj, uv, dir, obj, F, filter, T, spec, out, status, stream);
+    return launch_shade_s<false>(table, n_obj, uv, dir, obj, F, filter, T, spec, out, status, stream);
 }
 
 template <int FILTER, bool TILED>
