@@ -252,87 +252,87 @@ __global__ void __launch_bounds__(kShadeThreads) multi_shade_lanes_kernel(const 
 }
 
 // The same when every object is a bit texture in clamp mode: one number per
-// lookup instead of four equal channels, and a row's two bits from one word.  Any S <= 32: a warp takes
-// 32 / S fragments, and an S that is not a power of two is summed in the order of
-// the samples.  Bound: issue (the direction's mapping and eight gathers a
-// lookup).  10 poses of 1080p, S = 4, quadrilinear on 2 x 1024^2 x 16^2 bits: 1.15 ms
-// with the general kernel, 0.75 ms here (64 % of issue slots; 9 to 12
-// blocks per SM 0.77 to 0.81).
+// lookup instead of four equal channels, a row's two bits from one word, and a
+// fragment per thread, its samples one after another with the next direction
+// loaded ahead (the validity test, the spatial axes and the bucket offsets are
+// then a fragment's, not a lookup's).  A power of two up to 32 samples is summed
+// as the tree of multi_shade_lanes_kernel, others in their order.  Bound: issue.
+// 10 poses of 1080p, S = 4, quadrilinear on 2 x 1024^2 x 16^2 bits: 1.12 ms with the
+// general kernel, 0.77 with a lane per lookup, 0.645 here; 2 views of 1366 x 768
+// (lane per lookup -> here): S = 3, angular 56 -> 36 us, S = 16, quadrilinear 351 -> 265.
 template <int FILTER, int KIND>
 __global__ void __launch_bounds__(kShadeThreads, 8) multi_bits_kernel(const TexDesc* __restrict__ table, int n_obj,
                                                                       const float* __restrict__ uv,
                                                                       const float* __restrict__ dirs, int S,
                                                                       const int32_t* __restrict__ obj, int64_t F,
                                                                       float* __restrict__ out, unsigned* status) {
-    constexpr unsigned kAll = 0xffffffffu;
-    const int lane = threadIdx.x & 31, per = 32 / S;
-    const int g = lane / S, k = lane - g * S;  // this lane's fragment and sample of the warp's step
-    const bool used = g < per, pow2 = (S & (S - 1)) == 0;
-    const unsigned group = used ? (S == 32 ? kAll : ((1u << S) - 1u) << (g * S)) : 0u;
-    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * per;
     const float inv = 1.0f / (float)S;
-    float2 q = make_float2(0.f, 0.f);
-    float ix = 0.f, iy = 0.f, iz = 0.f;
-    int32_t o = -1;
-    auto fetch = [&](int64_t f) {
-        o = -1;
-        if (used && f < F) {
-            q = reinterpret_cast<const float2*>(uv)[f];
-            o = obj[f];
-            const float* I = dirs + 3 * (f * S + k);
-            ix = I[0];
-            iy = I[1];
-            iz = I[2];
+    const bool tree = S <= 32 && (S & (S - 1)) == 0;
+    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < F; f += (int64_t)gridDim.x * blockDim.x) {
+        const float2 q = reinterpret_cast<const float2*>(uv)[f];
+        const int32_t o = obj[f];
+        const float* I = dirs + 3 * (f * S);
+        float x = I[0], y = I[1], z = I[2];
+        float sum = 0.f, level[5];  // level[l]: the sum of the last whole left half of 2^l samples
+        bool ok = true;
+        for (int k = 0; k < S && ok; ++k) {
+            const float cx = x, cy = y, cz = z;
+            if (k + 1 < S) {
+                I += 3;
+                x = I[0];
+                y = I[1];
+                z = I[2];
+            }
+            TexDesc d;
+            ok = fragment_valid(table, n_obj, o, q.x, q.y, cx, cy, cz, status, d);
+            if (!ok) break;
+            const float c = filter_bits<FILTER, KIND>(d, locate<FILTER, false>(d, q.x, q.y, cx, cy, cz));
+            if (tree) {
+                sum = c;
+#pragma unroll
+                for (int l = 0; l < 5; ++l) {
+                    if (!((k >> l) & 1)) {
+                        level[l] = sum;
+                        break;
+                    }
+                    sum = level[l] + sum;
+                }
+            } else {
+                sum += c;
+            }
         }
-    };
-    fetch(warp0 * per + g);
-    for (int64_t base = warp0 * per; base < F; base += stride) {
-        const int64_t f = base + g;
-        const float2 cq = q;
-        const float cx = ix, cy = iy, cz = iz;
-        const int32_t co = o;
-        fetch(f + stride);
-        float c = 0.f;
-        bool bad = false;
-        TexDesc d;
-        if (fragment_valid(table, n_obj, co, cq.x, cq.y, cx, cy, cz, status, d))
-            c = filter_bits<FILTER, KIND>(d, locate<FILTER, false>(d, cq.x, cq.y, cx, cy, cz));
-        else
-            bad = co >= 0;  // an invalid sample zeroes its fragment
-        bad = (__ballot_sync(kAll, bad) & group) != 0;
-        if (pow2) {
-            for (int off = 1; off < S; off <<= 1) c += __shfl_xor_sync(kAll, c, off);
-        } else {
-            float sum = 0.f;
-            for (int m = 0; m < S; ++m) sum += __shfl_sync(kAll, c, g * S + m);
-            c = sum;
-        }
-        if (k == 0 && used && f < F) {
-            const float v = bad ? 0.f : c * inv;
-            __stcs(reinterpret_cast<float4*>(out) + f, make_float4(v, v, v, v));
-        }
+        const float v = ok ? sum * inv : 0.f;
+        __stcs(reinterpret_cast<float4*>(out) + f, make_float4(v, v, v, v));
     }
 }
 
 template <int FILTER, int KIND>
 static void launch_multi_bits(const TexDesc* table, int n_obj, const float* uv, const float* dirs, int S,
                               const int32_t* obj, int64_t F, float* out, unsigned* status, cudaStream_t stream) {
-    const unsigned grid = persistent_grid<multi_bits_kernel<FILTER, KIND>>(kShadeThreads, (F + 32 / S - 1) / (32 / S));
+    const unsigned grid = persistent_grid<multi_bits_kernel<FILTER, KIND>>(kShadeThreads, (F + 31) / 32);
     multi_bits_kernel<FILTER, KIND><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out, status);
 }
+
+// Below this many fragments a thread each leaves the chip (155 648 threads at 8
+// blocks per SM) idle while it walks its samples, and a lane per lookup is faster
+// where S divides a warp: 41 600 fragments, S = 16 (quadrilinear) 15.0 us against
+// 19.6, S = 8 9.1 against 11.4.  From some 60 000 to 95 000 on, by S and filter, the
+// thread per fragment wins (2.1 M: 265 us against 508).
+constexpr int64_t kFewFragments = 98304;
 
 template <int FILTER>
 static void launch_multi_t(const TexDesc* table, int n_obj, const float* uv, const float* dirs, int S,
                            const int32_t* obj, int64_t F, int bits, float* out, unsigned* status,
                            cudaStream_t stream) {
-    if (S <= 32 && bits == kBitsWords) {
+    const bool lanes = S <= 32 && (S & (S - 1)) == 0;
+    if (lanes && F < kFewFragments) bits = kBitsNone;
+    if (bits == kBitsWords) {
         launch_multi_bits<FILTER, kBitsWords>(table, n_obj, uv, dirs, S, obj, F, out, status, stream);
-    } else if (S <= 32 && bits == kBitsSmall) {
+    } else if (bits == kBitsSmall) {
         launch_multi_bits<FILTER, kBitsSmall>(table, n_obj, uv, dirs, S, obj, F, out, status, stream);
-    } else if (S <= 32 && bits == kBitsLarge) {
+    } else if (bits == kBitsLarge) {
         launch_multi_bits<FILTER, kBitsLarge>(table, n_obj, uv, dirs, S, obj, F, out, status, stream);
-    } else if (S <= 32 && (S & (S - 1)) == 0) {
+    } else if (lanes) {
         const unsigned grid = persistent_grid<multi_shade_lanes_kernel<FILTER>>(kShadeThreads, (F * S + 31) / 32);
         multi_shade_lanes_kernel<FILTER><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out,
                                                                               status);

@@ -90,3 +90,31 @@ def test_textures_of_2_to_the_32_texels_take_64_bit_indices():
     (a, ea), (b, eb) = _both([(65536, 16384, 2)], 0, uv, d, obj, api.RT_QUADRILINEAR, fill)
     np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
     assert ea == eb == api.RT_OK and 0.0 < a.mean() < 1.0
+
+
+@pytest.mark.parametrize("filt", FILTERS)
+@pytest.mark.parametrize("S", [1, 2, 4, 8, 16, 32])
+def test_many_fragments_sum_powers_of_two_as_the_lanes_do(filt, S):
+    """Enough fragments for a thread each: the samples' tree of sums is that of the lanes, bit for bit."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    uv, d, obj = _inputs(100003, S, S, 2)
+    (a, ea), (b, eb) = _both([(37, 23, 5), (64, 32, 8)], 5, uv, d, obj, filt)
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+    assert ea == eb == api.RT_OK and a.any()
+
+
+@pytest.mark.parametrize("filt", FILTERS)
+def test_64_bit_indices_a_thread_per_fragment(filt):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    uv, d, obj = _inputs(10007, 3, 4, 1)
+    obj[:] = 0
+    scene = synth.bake_scene(11)
+
+    def fill(ctx, oid):
+        api.rt_bake_shadow(ctx, oid, api.RT_SURFACE_PLANE, scene)
+
+    (a, ea), (b, eb) = _both([(65536, 16384, 2)], 0, uv, d, obj, filt, fill)
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+    assert ea == eb == api.RT_OK and 0.0 < a.mean() < 1.0
