@@ -66,12 +66,33 @@ __device__ __forceinline__ P4 quadrilinear_combine(const P4 (&q)[4][4], const Ax
     return lerpP(lerpP(c[0], c[1], wu), lerpP(c[2], c[3], wu), wv);
 }
 
+// The same from FP16 / BF16 codes, bit for bit.
+template <int FMT>
+__device__ __forceinline__ P4 quadrilinear_combine_codes(const uint2 (&q)[4][4], const Axis& U, const Axis& V,
+                                                         const Axis& S, const Axis& T) {
+    const f32x2 ws = pack2(S.w, S.w), wt = pack2(T.w, T.w), wu = pack2(U.w, U.w), wv = pack2(V.w, V.w);
+    P4 c[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+        c[b] = lerpP(lerp8<FMT>(q[b][0], q[b][1], ws), lerp8<FMT>(q[b][2], q[b][3], ws), wt);
+    return lerpP(lerpP(c[0], c[1], wu), lerpP(c[2], c[3], wu), wv);
+}
+
 template <int FMT, int LAYOUT>
 __device__ __forceinline__ P4 quadrilinear_planes(const TexDesc& d, const Axis& U, const Axis& V, const Axis& S,
                                                   const Axis& T) {
     int64_t pl[4];
     int o[4];
     quad_tap_addresses<LAYOUT>(d, U, V, S, T, pl, o);
+    if constexpr (FMT == RT_F16 || FMT == RT_BF16) {
+        uint2 code[4][4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                code[b][k] = __ldg(reinterpret_cast<const uint2*>(d.base) + checked_texel(d, pl[k] + o[b]));
+        return quadrilinear_combine_codes<FMT>(code, U, V, S, T);
+    }
     float sc[4] = {1.f, 1.f, 1.f, 1.f};
     if (FMT == RT_E4M3_BUCKET_SCALE) {
 #pragma unroll

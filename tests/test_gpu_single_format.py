@@ -105,3 +105,22 @@ def test_world_backward(pair, fmt, palette):
             for k in oids:
                 assert bool(((at[k] - bt[k]).abs() <= 1e-4 * weight[k]).all())
     assert api.rt_get_error(pair[0]) == api.RT_OK
+
+
+@pytest.mark.parametrize("fmt,dtype", [(api.RT_F16, torch.float16), (api.RT_BF16, torch.bfloat16)])
+def test_16_bit_codes_shade_as_their_values(pair, fmt, dtype):
+    """An FP16 / BF16 texture shades, bit for bit, as an FP32 one of the same values: widening is
+    exact.  Random codes: every magnitude, subnormals, infinities (no NaN)."""
+    W, H, n = 37, 23, 8
+    rng = np.random.default_rng(11)
+    codes = torch.from_numpy(rng.integers(-32768, 32768, (n, n, H, W, 4)).astype(np.int16)).view(dtype)
+    values = torch.where(codes.isnan(), torch.zeros_like(codes), codes).float().to("cuda")
+    for c, f in ((pair[0], fmt), (pair[1], api.RT_F32)):
+        api.rt_create_texture(c, W, H, n, f, api.RT_LAYOUT_PLANES, values)
+        api.rt_create_texture(c, W, H, n, f, api.RT_LAYOUT_PLANES, values.flip(2))
+    for shape in SHAPES:
+        uv, d, N, o = frames(shape, [0, 1])
+        for filt in FILTERS:
+            a, b = (torch.stack([api.rt_shade_batched(c, uv, d, o, filt),
+                                 api.rt_shade_world_batched(c, uv, d, N, o, filt)]) for c in pair)
+            assert torch.allclose(a, b, rtol=0.0, atol=0.0, equal_nan=True)
