@@ -430,8 +430,8 @@ __device__ __forceinline__ P4 decode8<RT_BF16>(uint2 r) {
 }
 
 // a + w (b - a) of two 8-byte FP16 / BF16 codes: b is subtracted unwidened (sub
-// of a 16-bit and an FP32 operand, sm_100 and later), the same roundings with a
-// quarter of the conversions.  The forward is bound by issue: 20 poses of 1080p
+// of a 16-bit and an FP32 operand, sm_100 and later), the same roundings with
+// half of the conversions.  The forward is bound by issue: 20 poses of 1080p
 // FP16 0.503 -> 0.480 ms, 64 objects on two 4K frames 0.303 -> 0.276, the
 // world-space lookup with its gradients 0.836 -> 0.805; in the fused step the same
 // gave 0.5 %, within its runs' spread, so that one widens every code.
