@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kBackThreads, DET ? 4 : (TILED && SPEC >= 0) ?
             if (any_grad) grad = grads.p[q.o];
         }
         if (DET) {
-            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
+            reduce_fixed_warp<FILTER, SPEC>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
             grad = nullptr;
         }
         if (valid && (!DET || coord_grads)) {
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kBackThreads, SPEC >= 0 ? 6 : 1) world_backwar
             if (any_grad) grad = grads.p[q.o];
         }
         if (DET) {
-            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
+            reduce_fixed_warp<FILTER, SPEC>(valid && grad && d.fmt != RT_BIT1, d, L, go, grad, status);
             grad = nullptr;
         }
         if (valid && (!DET || coord_grads)) {

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kBackThreads, (DET || SPEC >= 0) ? 4 : 1) fuse
                                      scale * (c.w - t.w));
         void* grad = valid && any_grad ? grads.p[q.o] : nullptr;
         if (DET) {
-            reduce_fixed_warp<FILTER>(valid && grad && d.fmt != RT_BIT1, d, L, g, grad, status);
+            reduce_fixed_warp<FILTER, SPEC>(valid && grad && d.fmt != RT_BIT1, d, L, g, grad, status);
             grad = nullptr;
         }
         if (valid && (!DET || coord_grads)) {

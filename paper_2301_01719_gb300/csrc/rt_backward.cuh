@@ -98,7 +98,8 @@ __device__ __forceinline__ void tap_table(const TexDesc& d, const Lookup<FILTER>
 // 1.63 ms to 0.60 ms; adding the texels that horizontal neighbours share once (as
 // reduce_quadrilinear_taps does) took 0.94 ms, the partner's weights costing
 // more than the adds they save.
-template <int FILTER>
+// SPEC as in filter_spec: >= 0 where no object can be in the ATLAS layout.
+template <int FILTER, int SPEC>
 __device__ __forceinline__ void reduce_fixed_warp(bool has, const TexDesc& d, const Lookup<FILTER>& L, float4 g,
                                                   void* grad, unsigned* status) {
     constexpr unsigned kAll = 0xffffffffu;
@@ -109,7 +110,7 @@ __device__ __forceinline__ void reduce_fixed_warp(bool has, const TexDesc& d, co
 #pragma unroll 1
     for (int r = 0; r < 4; ++r) {
         const int src = (lane & 28) | r;
-        const bool hr = __shfl_sync(kAll, (int)has, src) != 0;
+        const int hr = __shfl_sync(kAll, (has ? 1 : 0) | (SPEC < 0 && has && d.layout == RT_LAYOUT_ATLAS ? 2 : 0), src);
         char* base = reinterpret_cast<char*>(__shfl_sync(kAll, (unsigned long long)grad, src)) + 8 * c;
         const float gx = __shfl_sync(kAll, g.x, src), gy = __shfl_sync(kAll, g.y, src);
         const float gz = __shfl_sync(kAll, g.z, src), gw = __shfl_sync(kAll, g.w, src);
@@ -138,7 +139,7 @@ __device__ __forceinline__ void reduce_fixed_warp(bool has, const TexDesc& d, co
 #ifdef RADTEX_CHECKED
         const int64_t extent = __shfl_sync(kAll, has ? d.extent : (int64_t)0, src);
 #endif
-        if (!hr) continue;
+        if (hr == 0) continue;
         auto add = [&](int b, int k, unsigned long long v) {
             int64_t idx = ob[b] + ot[k];
 #ifdef RADTEX_CHECKED
@@ -151,11 +152,19 @@ __device__ __forceinline__ void reduce_fixed_warp(bool has, const TexDesc& d, co
         };
         // the weights lie in [0, 1], so |g| decides for every contribution
         const bool small = fabsf(gc) <= kFixedSmall;
+        // a tap's weight is rounded as the FP32 reductions round it: (wb ws) wt, and wb (ws wt)
+        // in the ATLAS layout
         float w[T.kBuckets][T.kTexels];
 #pragma unroll
         for (int b = 0; b < T.kBuckets; ++b)
 #pragma unroll
             for (int k = 0; k < T.kTexels; ++k) w[b][k] = wb[b] * ws[k & 1] * wt[k >> 1];
+        if (SPEC < 0 && FILTER == RT_QUADRILINEAR && (hr & 2)) {
+#pragma unroll
+            for (int b = 0; b < T.kBuckets; ++b)
+#pragma unroll
+                for (int k = 0; k < T.kTexels; ++k) w[b][k] = wb[b] * (ws[k & 1] * wt[k >> 1]);
+        }
         if (small) {
 #pragma unroll
             for (int b = 0; b < T.kBuckets; ++b)
