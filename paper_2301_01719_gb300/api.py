@@ -245,11 +245,11 @@ def palette_encode(ctx: Context, obj_id: int, K: int, iterations: int, seed: int
         else:
             rt_kmeans_reassign_tc(ctx, obj_id, K, C, index, dist, tc, stream=stream)
 
-    for step in range(iterations):
-        assign(step == 0)
+    for _ in range(iterations):
+        assign(not sse)
         sse.append(dist.sum(dtype=torch.float64))
         rt_kmeans_update(ctx, obj_id, K, index, C, scratch, stream=stream)
-    assign(iterations == 0)
+    assign(not sse)
     sse.append(dist.sum(dtype=torch.float64))
     return C, index, torch.stack(sse).tolist()
 
