@@ -218,19 +218,39 @@ def rt_kmeans_update(ctx: Context, obj_id: int, K: int, index: torch.Tensor, cen
     return centroids
 
 
+def _torch_stream(stream, device) -> torch.cuda.Stream:
+    """A stream argument (torch stream, object with a cuda_stream handle, or raw handle) as a torch stream."""
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    handle = _stream(stream, device)
+    if handle in (0, 1):  # the legacy default stream
+        return torch.cuda.default_stream(device)
+    return torch.cuda.ExternalStream(handle, device=device)
+
+
 def palette_encode(ctx: Context, obj_id: int, K: int, iterations: int, seed: int = 0, stream=None,
                    tensor_cores: bool = True):
     """k-means palette of a dense texture: K centroids seeded at K distinct random
     buckets, `iterations` Lloyd steps, assignments on the tensor cores (FP16
     operands) unless tensor_cores is False (FP32 on the CUDA cores).  Returns
-    (centroids (n, n, K, 4), index (h, w), per-step sums of squared distances)."""
-    import numpy as np
-
+    (centroids (n, n, K, 4), index (h, w), per-step sums of squared distances).
+    With a stream, all of it runs there, after the current stream's work so far; it is
+    done when the call returns."""
+    dev = torch.device("cuda", ctx.device)
+    if stream is not None:
+        # the sums of the distances and every buffer belong to the stream too: on the current one they
+        # would race with the kernels
+        current, stream = torch.cuda.current_stream(dev), _torch_stream(stream, dev)
+        stream.wait_stream(current)
+        with torch.cuda.stream(stream):
+            C, index, sse = palette_encode(ctx, obj_id, K, iterations, seed, tensor_cores=tensor_cores)
+        C.record_stream(current)
+        index.record_stream(current)
+        return C, index, sse
     info = rt_texture_info(ctx, obj_id)
     B = info["w"] * info["h"]
-    dev = torch.device("cuda", ctx.device)
     pick = np.random.default_rng(seed).choice(B, size=K, replace=False).astype(np.int32)
-    C = rt_kmeans_init(ctx, obj_id, K, torch.from_numpy(pick).to(dev), stream=stream)
+    C = rt_kmeans_init(ctx, obj_id, K, torch.from_numpy(pick).to(dev))
     scratch = torch.empty(B + 3 * K + 1, dtype=torch.int32, device=dev)
     index = torch.empty((info["h"], info["w"]), dtype=torch.int32, device=dev)
     dist = torch.empty((info["h"], info["w"]), dtype=torch.float32, device=dev)
@@ -239,16 +259,16 @@ def palette_encode(ctx: Context, obj_id: int, K: int, iterations: int, seed: int
 
     def assign(first):
         if not tensor_cores:
-            rt_kmeans_assign(ctx, obj_id, K, C, index, dist, stream=stream)
+            rt_kmeans_assign(ctx, obj_id, K, C, index, dist)
         elif first:
-            rt_kmeans_assign_tc(ctx, obj_id, K, C, index, dist, scratch=tc, stream=stream)
+            rt_kmeans_assign_tc(ctx, obj_id, K, C, index, dist, scratch=tc)
         else:
-            rt_kmeans_reassign_tc(ctx, obj_id, K, C, index, dist, tc, stream=stream)
+            rt_kmeans_reassign_tc(ctx, obj_id, K, C, index, dist, tc)
 
     for _ in range(iterations):
         assign(not sse)
         sse.append(dist.sum(dtype=torch.float64))
-        rt_kmeans_update(ctx, obj_id, K, index, C, scratch, stream=stream)
+        rt_kmeans_update(ctx, obj_id, K, index, C, scratch)
     assign(not sse)
     sse.append(dist.sum(dtype=torch.float64))
     return C, index, torch.stack(sse).tolist()

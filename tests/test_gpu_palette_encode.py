@@ -38,3 +38,29 @@ def test_a_negative_number_of_steps_is_none(ctx, oid, tensor_cores):
     for steps in (-1, -5):
         torch.full((1 << 22,), float("nan"), device="cuda")  # what the scratch may be given next
         assert same(api.palette_encode(ctx, oid, K, steps, tensor_cores=tensor_cores), none)
+
+
+@pytest.mark.parametrize("tensor_cores", [True, False])
+@pytest.mark.parametrize("busy", ["given", "current"])
+@pytest.mark.parametrize("kind", ["torch", "handle"])
+def test_a_given_stream_runs_the_whole_encoding(ctx, oid, tensor_cores, busy, kind):
+    """With work queued on either stream (some 20 ms of fills), an encoding on a side stream equals the
+    one on the current stream: its sums are taken after each assignment and before the next."""
+    want = api.palette_encode(ctx, oid, K, 3, seed=2, tensor_cores=tensor_cores)
+    side = torch.cuda.Stream()
+    filler = torch.empty(1 << 28, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side if busy == "given" else torch.cuda.current_stream()):
+        for k in range(100):
+            filler.fill_(float(k))
+    got = api.palette_encode(ctx, oid, K, 3, seed=2, stream=side if kind == "torch" else side.cuda_stream,
+                             tensor_cores=tensor_cores)
+    assert same(got, want)
+    torch.cuda.synchronize()
+
+
+def test_the_default_streams_handle_is_a_stream_too(ctx, oid):
+    want = api.palette_encode(ctx, oid, K, 1)
+    assert same(api.palette_encode(ctx, oid, K, 1, stream=0), want)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        assert same(api.palette_encode(ctx, oid, K, 1, stream=torch.cuda.default_stream()), want)
