@@ -145,9 +145,11 @@ static cudaError_t launch_relayout(const void* src, int src_layout, void* dst, i
                                    cudaStream_t stream) {
     const S* s = static_cast<const S*>(src);
     D* d = static_cast<D*>(dst);
-    if (W >= kTileMinWidth) {
-        const RelayoutShape r = relayout_shape(W, H, n);
-        // w h <= 2^30 (or a K x 1 palette, K <= 2^30) and n <= 64: at most 2^25 x 256 blocks
+    const RelayoutShape r = relayout_shape(W, H, n);
+    // a texture's n is at most 64, but an FP32 buffer to convert may have more in-bucket rows and chunks of
+    // columns than a grid has in y (n = 1024 and on)
+    if (W >= kTileMinWidth && (int64_t)n * r.chunks <= 65535) {
+        // w h <= 2^30 (or a K x 1 palette, K <= 2^30) for a texture: at most 2^25 blocks in x
         const dim3 grid((unsigned)r.ti * (unsigned)r.tj, (unsigned)(n * r.chunks));
         relayout_tiles<S, D, Op><<<grid, kThreads, 0, stream>>>(s, src_layout, d, dst_layout, r);
     } else {

@@ -68,3 +68,16 @@ def test_stored_codes_read_back_in_every_layout(ctx, w, h, n, storage):
             got = api.rt_read_texture(ctx, oid, dst)[0].cpu().numpy()
             np.testing.assert_array_equal(got, _in_layout(want, dst, w, h, n))
         api.rt_destroy_texture(ctx, oid)
+
+
+@pytest.mark.parametrize("w,n", [(24, 1023), (24, 1024), (23, 1024)])
+def test_convert_layout_of_many_in_bucket_texels(w, n):
+    """rt_convert_layout has no limit on n; a grid has one on its second dimension (reached at n = 1024)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    a = torch.arange(n * n * w * 4, dtype=torch.int32, device="cuda").view(n, n, 1, w, 4)
+    planes = a.view(torch.float32)  # distinct bit patterns
+    got = api.rt_convert_layout(planes, api.RT_LAYOUT_PLANES, api.RT_LAYOUT_ATLAS, w, 1, n)
+    assert torch.equal(got.view(torch.int32), a[:, :, 0].permute(0, 2, 1, 3).reshape(n, w * n, 4))
+    back = api.rt_convert_layout(got, api.RT_LAYOUT_ATLAS, api.RT_LAYOUT_PLANES, w, 1, n)
+    assert torch.equal(back.view(torch.int32), a)
