@@ -123,8 +123,7 @@ __global__ void __launch_bounds__(kThreads, 6) relayout_tiles(const S* __restric
     for_tile_texels(dst_layout, r, i0, j0, t, s0, [&](int64_t o, int p) { dst[o] = tile[p]; });
 }
 
-// One thread per texel in plane order, for narrow bucket matrices, which leave
-// most of a tile empty.
+// One thread per texel in plane order, for copies that leave most of a tile empty.
 template <typename S, typename D, typename Op>
 __global__ void relayout_texels(const S* __restrict__ src, int src_layout, D* __restrict__ dst, int dst_layout, int W,
                                 int H, int n, int64_t total) {
@@ -135,10 +134,32 @@ __global__ void relayout_texels(const S* __restrict__ src, int src_layout, D* __
     dst[index_in(dst_layout, W, H, n, i, j, s, t)] = Op()(src[index_in(src_layout, W, H, n, i, j, s, t)]);
 }
 
-// FP32, 2^17 buckets x 16^2, tiles against one thread per texel: 16 wide 311 /
-// 476 us (QUADS to ATLAS) but 258 / 195 us (PLANES to QUADS), 24 wide 164 / 472
-// and 159 / 195, 8 wide 545 / 492 and 473 / 195.
-constexpr int kTileMinWidth = 24;
+// Tiles, or a thread per texel.  A block's costs are those of a whole tile (64
+// buckets x 16 columns), so it must hold enough of them: bucket rows of 24 and
+// more, and 8 columns where the tile has two bucket rows, 16 where the matrix has
+// one (a palette).  Tiles / texels in us, all pairs of layouts, on 2^20 to 2^23
+// texels of FP32, 2-byte and E4M3 channels:
+//   width (FP32, 2^17 buckets x 16^2), QUADS to ATLAS and PLANES to QUADS: 8 wide
+//     545 / 492 and 473 / 195, 16 wide 311 / 476 and 258 / 195, 24 wide 164 / 472 and 159 / 195;
+//   columns n: n = 1, 2, 4 are 4-6, 2-3 and 1.2-1.7 times as slow in tiles (1000 x 2097 x 2^2 FP32
+//     PLANES to QUADS 149 / 72), n = 8 0.5-1.2 times, n = 16 0.4-1.0 (copies within one layout
+//     0.5-0.9);
+//   one bucket row: n = 8 1.0-1.4 times as slow, n = 12 0.7-1.1, n = 16 0.7-1.0, n = 17 (chunks of
+//     9) 1.0-1.4.
+// FP32 texels into an ATLAS, which a thread per texel stores one by one past L2,
+// are faster in tiles from 5 columns on where the copy outgrows L2: 256 x 1310 x
+// 5^2 from QUADS 68 / 100, 64 x 1820 x 6^2 33 / 33, 256 x 910 x 6^2 60 / 87.
+constexpr int kTileMinWidth = 24, kTileMinColumns = 8;
+
+static bool tiles_pay(const RelayoutShape& r, bool fp32_to_atlas) {
+    // a texture's n is at most 64, but an FP32 buffer to convert may have more in-bucket rows and
+    // chunks of columns than a grid has in y (n = 1024 and on)
+    if (r.W < kTileMinWidth || (int64_t)r.n * r.chunks > 65535) return false;
+    if (r.H == 1) return r.sc == kTileS;
+    if (r.sc >= kTileMinColumns) return true;
+    const int64_t texels = (int64_t)r.W * r.H * r.n * r.n;
+    return fp32_to_atlas && r.sc >= 5 && texels >= (r.sc == 5 ? (int64_t)1 << 23 : (int64_t)1 << 22);
+}
 
 template <typename S, typename D, typename Op = CopyTexel>
 static cudaError_t launch_relayout(const void* src, int src_layout, void* dst, int dst_layout, int W, int H, int n,
@@ -146,9 +167,7 @@ static cudaError_t launch_relayout(const void* src, int src_layout, void* dst, i
     const S* s = static_cast<const S*>(src);
     D* d = static_cast<D*>(dst);
     const RelayoutShape r = relayout_shape(W, H, n);
-    // a texture's n is at most 64, but an FP32 buffer to convert may have more in-bucket rows and chunks of
-    // columns than a grid has in y (n = 1024 and on)
-    if (W >= kTileMinWidth && (int64_t)n * r.chunks <= 65535) {
+    if (tiles_pay(r, sizeof(D) == 16 && dst_layout == RT_LAYOUT_ATLAS)) {
         // w h <= 2^30 (or a K x 1 palette, K <= 2^30) for a texture: at most 2^25 blocks in x
         const dim3 grid((unsigned)r.ti * (unsigned)r.tj, (unsigned)(n * r.chunks));
         relayout_tiles<S, D, Op><<<grid, kThreads, 0, stream>>>(s, src_layout, d, dst_layout, r);

@@ -81,3 +81,27 @@ def test_convert_layout_of_many_in_bucket_texels(w, n):
     assert torch.equal(got.view(torch.int32), a[:, :, 0].permute(0, 2, 1, 3).reshape(n, w * n, 4))
     back = api.rt_convert_layout(got, api.RT_LAYOUT_ATLAS, api.RT_LAYOUT_PLANES, w, 1, n)
     assert torch.equal(back.view(torch.int32), a)
+
+
+@pytest.mark.parametrize("w,h,n", [(40, 3, 7), (40, 3, 8), (24, 2, 8), (23, 2, 8), (40, 1, 15), (40, 1, 16), (40, 1, 17),
+                                   (40, 1, 31), (40, 1, 32), (40, 2, 5), (64, 1820, 6), (64, 1821, 6), (100, 3355, 5),
+                                   (100, 3356, 5)])
+def test_copies_on_both_sides_of_the_tiles_rule(ctx, w, h, n):
+    """Every pair of layouts where tiles begin and end (widths, in-bucket columns, one bucket row, large
+    FP32 copies into an atlas), and the FP16 codes of the same sizes."""
+    planes = torch.arange(n * n * w * h * 4, dtype=torch.int32, device="cuda").view(n, n, h, w, 4)
+    atlas = planes.permute(2, 0, 3, 1, 4).reshape(h * n, w * n, 4)
+    full = torch.full((n, n, h + h % 2, w + w % 2, 4), -7, dtype=torch.int32, device="cuda")
+    full[:, :, :h, :w] = planes
+    quads = full.view(n, n, full.shape[2] // 2, 2, full.shape[3] // 2, 2, 4).transpose(3, 4).contiguous()
+    held = {api.RT_LAYOUT_ATLAS: atlas.contiguous(), api.RT_LAYOUT_PLANES: planes, api.RT_LAYOUT_QUADS: quads}
+    for src in LAYOUTS:
+        for dst in LAYOUTS:
+            to = torch.full(held[dst].shape, -7, dtype=torch.int32, device="cuda").view(torch.float32)
+            api.rt_convert_layout(held[src].view(torch.float32), src, dst, w, h, n, to)
+            assert torch.equal(to.view(torch.int32), held[dst])
+    values = (atlas % 2039).float()  # exact in FP16
+    oid = api.rt_create_texture(ctx, w, h, n, api.RT_F16, api.RT_LAYOUT_ATLAS, values)
+    for dst, want in ((api.RT_LAYOUT_ATLAS, values), (api.RT_LAYOUT_PLANES, (planes % 2039).float())):
+        assert torch.equal(api.rt_read_texture(ctx, oid, dst)[0].view(torch.float16).float(), want)
+    api.rt_destroy_texture(ctx, oid)
