@@ -315,12 +315,14 @@ __global__ void __launch_bounds__(THREADS, 1)
 // the last plane are zeros; the rows beyond the last bucket are not written (a
 // row only reaches its own distances, which are not stored).  On 512^2 x 16^2
 // FP16: 0.29 ms by blocks of 32 buckets x 8 planes and 0.08 ms for a pass of X
-// that took the norms; 0.20 ms for both.
+// that took the norms; 0.20 ms for both.  Few buckets with many planes leave
+// the chip idle while each block walks its planes: then (SPLIT) gridDim.y blocks
+// take `share` planes each, and a pass over X takes the norms.
 constexpr int CI = 16, CJ = 2, CB = CI * CJ, CP = 64, CTHREADS = 256;
 
-template <int FMT, int LAYOUT>
-__global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, __half* __restrict__ X,
-                                                             float* __restrict__ xn) {
+template <int FMT, int LAYOUT, bool SPLIT>
+__global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, int share,
+                                                             __half* __restrict__ X, float* __restrict__ xn) {
     __shared__ uint2 tile[CP][CB + 1];
     const int planes = d.n * d.n, P4 = Dp / 4, ti = (d.W + CI - 1) / CI;
     const int tj = (int)(blockIdx.x / (unsigned)ti), i0 = (int)(blockIdx.x - (unsigned)tj * ti) * CI, j0 = tj * CJ;
@@ -339,7 +341,8 @@ __global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, 
     float norm[CB / (CTHREADS / 32)];
 #pragma unroll
     for (int r = 0; r < CB / (CTHREADS / 32); ++r) norm[r] = 0.0f;
-    for (int p0 = 0; p0 < P4; p0 += CP) {
+    const int p_first = SPLIT ? (int)blockIdx.y * share : 0, p_end = SPLIT ? min(p_first + share, P4) : P4;
+    for (int p0 = p_first; p0 < p_end; p0 += CP) {
 #pragma unroll
         for (int k = 0; k < CP / (CTHREADS / 32); ++k) {
             const int q = warp + k * (CTHREADS / 32), p = p0 + q;
@@ -375,6 +378,7 @@ __global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, 
         }
         __syncthreads();
     }
+    if (SPLIT) return;
 #pragma unroll
     for (int r = 0; r < CB / (CTHREADS / 32); ++r) {
         float s = norm[r];
@@ -385,7 +389,7 @@ __global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, 
     }
 }
 
-// |c_k|^2 of the FP16 rows (one warp per centroid).
+// |x|^2 of FP16 rows (one warp per row): the centroids', and the buckets' where the conversion is split.
 __global__ void row_norms_kernel(const __half* __restrict__ X, int rows, int Dp, float* __restrict__ out,
                                  float pad_value, int live_rows) {
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -467,10 +471,30 @@ static bool make_map(CUtensorMap* m, void* ptr, int64_t rows, int64_t cols, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Fewer blocks than kSplitBelow (2 per SM) split their planes, from kSplitGroups
+// groups of CP planes on, into about kSplitInto blocks.  One assignment with K = 16,
+// FP16, whole / split in us: 16^2 x 64^2 buckets 220 / 113, 64^2 x 64^2 (128 blocks) 403 / 217, 64^2 x
+// 16^2 32.8 / 31.0, 120 x 64 x 16^2 (240) 34.5 / 34.5; but 100^2 x 16^2 (350) 35 / 39, 128^2 x 32^2
+// (512) 138 / 145, and with 2 groups 33 x 200 x 9^2 26.6 / 28.7: the norms' pass costs
+// more than the split gives.  64^2 x 64^2 into 304, 608 and 1216 blocks: 242, 249, 217.
+constexpr unsigned kSplitBelow = 304, kSplitInto = 1216, kSplitGroups = 4;
+
 template <int FMT, int LAYOUT>
 static cudaError_t convert_x(const TexDesc& d, const Layout& L, __half* X, float* xn, cudaStream_t stream) {
-    const unsigned grid = (unsigned)((d.W + CI - 1) / CI) * (unsigned)((d.H + CJ - 1) / CJ);
-    convert_x_kernel<FMT, LAYOUT><<<grid, CTHREADS, 0, stream>>>(d, (int)L.Dp, X, xn);
+    const unsigned blocks = (unsigned)((d.W + CI - 1) / CI) * (unsigned)((d.H + CJ - 1) / CJ);
+    const unsigned groups = (unsigned)((L.Dp / 4 + CP - 1) / CP);
+    unsigned split = groups >= kSplitGroups && blocks < kSplitBelow ? (kSplitInto + blocks - 1) / blocks : 1;
+    if (split > groups) split = groups;
+    const unsigned each = (groups + split - 1) / split;  // groups per block
+    split = (groups + each - 1) / each;
+    if (split > 1) {
+        convert_x_kernel<FMT, LAYOUT, true><<<dim3(blocks, split), CTHREADS, 0, stream>>>(d, (int)L.Dp,
+                                                                                          (int)each * CP, X, xn);
+        row_norms_kernel<<<(unsigned)((L.Bp * 32 + 255) / 256), 256, 0, stream>>>(X, d.W * d.H, (int)L.Dp, xn, 0.f,
+                                                                                  d.W * d.H);
+    } else {
+        convert_x_kernel<FMT, LAYOUT, false><<<blocks, CTHREADS, 0, stream>>>(d, (int)L.Dp, 0, X, xn);
+    }
     return cudaGetLastError();
 }
 

@@ -112,3 +112,25 @@ def test_tensor_core_assignment_and_reassignment(ctx, w, h, n, K, storage, layou
     assert api.rt_get_error(ctx) == api.RT_OK
     api.rt_destroy_texture(ctx, oid)
     del keep
+
+
+@pytest.mark.parametrize("w,h,n,K", [(8, 8, 16, 5), (9, 5, 17, 3), (16, 16, 15, 4), (5, 3, 33, 2), (16, 16, 64, 16),
+                                     (160, 59, 16, 7),
+                                     (160, 61, 16, 7)])
+@pytest.mark.parametrize("storage,layout,flags", KINDS)
+def test_tensor_core_distances_of_few_buckets_with_many_planes(ctx, w, h, n, K, storage, layout, flags):
+    """The conversion of few buckets (160 x 61 are the first with enough) splits their planes among blocks,
+    from 4 groups of 64 planes on, groups that the split does not divide among them: indices and distances within the documented bound."""
+    rng = np.random.default_rng(w + h + n)
+    oid, keep, X = _texture(ctx, rng.uniform(-1.0, 1.0, (n, n, h, w, 4)).astype(np.float32), storage, layout, flags)
+    C = rng.uniform(-1.0, 1.0, (n, n, K, 4)).astype(np.float32)
+    index, dist = api.rt_kmeans_assign_tc(ctx, oid, K, torch.from_numpy(C).cuda(), want_dist=True)
+    C = C.astype(np.float64).reshape(n * n, K, 4).transpose(1, 0, 2).reshape(K, -1)
+    D = (X ** 2).sum(1)[:, None] + (C ** 2).sum(1)[None] - 2.0 * X @ C.T
+    bound = 2.0 ** -10 * ((X ** 2).sum(1) + (C ** 2).sum(1).max())
+    got = D[np.arange(w * h), index.cpu().numpy().reshape(-1)]
+    assert (got <= D.min(1) + bound).all()
+    assert (np.abs(dist.cpu().numpy().reshape(-1) - got) <= bound).all()
+    assert api.rt_get_error(ctx) == api.RT_OK
+    api.rt_destroy_texture(ctx, oid)
+    del keep
