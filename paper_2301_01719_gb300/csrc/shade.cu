@@ -313,19 +313,31 @@ static void launch_multi_bits(const TexDesc* table, int n_obj, const float* uv, 
     multi_bits_kernel<FILTER, KIND><<<grid, kShadeThreads, 0, stream>>>(table, n_obj, uv, dirs, S, obj, F, out, status);
 }
 
-// Below this many fragments a thread each leaves the chip (155 648 threads at 8
-// blocks per SM) idle while it walks its samples, and a lane per lookup is faster
-// where S divides a warp: 41 600 fragments, S = 16 (quadrilinear) 15.0 us against
-// 19.6, S = 8 9.1 against 11.4.  From some 60 000 to 95 000 on, by S and filter, the
-// thread per fragment wins (2.1 M: 265 us against 508).
-constexpr int64_t kFewFragments = 98304;
+// Below this many fragments a lane per lookup is faster where S divides a warp: a
+// thread per fragment leaves the chip (155 648 threads at 8 blocks per SM) or its
+// last round partly idle for as long as the samples of a fragment take, and the
+// cheaper filters gain less from sharing the fragment's work.  Thread / lane, 1024 x
+// 512 x 16^2 bits, every fragment with an object, S = 4, 8, 16, 32:
+//   quadrilinear: 60 000 fragments 1.00, 0.86, 0.93, 1.00, 98 304 0.75, 0.73, 0.81, 0.91, 1.5 M 0.59,
+//     0.54, 0.58, 0.67;
+//   angular-bilinear: 60 000 1.00, 1.07, 1.14, 1.46, 98 304 0.75, 0.83, 1.00, 1.31, 200 000 0.83, 0.85, 1.05,
+//     1.27, 250 000 0.72, 0.77, 0.97, 1.16, 480 000 0.67, 0.67, 0.85, 1.07, 1.5 M 0.60, 0.58, 0.78, 1.00
+//     (with the background of a frame among them 0.91);
+//   nearest: 98 304 1.00, 0.93, 1.00, 1.41, 200 000 0.84, 0.88, 1.08, 1.37, 250 000 0.83, 0.73, 1.00, 1.25, 1.5 M
+//     0.63, 0.62, 0.86, 1.13.
+template <int FILTER>
+static int64_t few_fragments(int S) {
+    if (FILTER == RT_QUADRILINEAR || S < 16) return 98304;
+    if (S == 16) return 262144;
+    return FILTER == RT_NEAREST ? INT64_MAX : 524288;
+}
 
 template <int FILTER>
 static void launch_multi_t(const TexDesc* table, int n_obj, const float* uv, const float* dirs, int S,
                            const int32_t* obj, int64_t F, int bits, float* out, unsigned* status,
                            cudaStream_t stream) {
     const bool lanes = S <= 32 && (S & (S - 1)) == 0;
-    if (lanes && F < kFewFragments) bits = kBitsNone;
+    if (lanes && F < few_fragments<FILTER>(S)) bits = kBitsNone;
     if (bits == kBitsWords) {
         launch_multi_bits<FILTER, kBitsWords>(table, n_obj, uv, dirs, S, obj, F, out, status, stream);
     } else if (bits == kBitsSmall) {

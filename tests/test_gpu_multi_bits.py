@@ -118,3 +118,23 @@ def test_64_bit_indices_a_thread_per_fragment(filt):
     (a, ea), (b, eb) = _both([(65536, 16384, 2)], 0, uv, d, obj, filt, fill)
     np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
     assert ea == eb == api.RT_OK and 0.0 < a.mean() < 1.0
+
+
+WORDS = [(64, 32, 8), (37, 32, 3), (1, 32, 2)]  # planes of whole words
+ANY = [(37, 23, 5), (64, 32, 8), (1, 1, 1)]
+
+
+@pytest.mark.parametrize("sizes", [WORDS, ANY])
+@pytest.mark.parametrize("S,filt,F", [
+    (4, api.RT_QUADRILINEAR, 98303), (4, api.RT_QUADRILINEAR, 98304), (8, api.RT_NEAREST, 98304),
+    (16, api.RT_QUADRILINEAR, 98304), (16, api.RT_NEAREST, 262143), (16, api.RT_NEAREST, 262144),
+    (16, api.RT_ANGULAR_BILINEAR, 262144), (32, api.RT_ANGULAR_BILINEAR, 524287),
+    (32, api.RT_ANGULAR_BILINEAR, 524288), (32, api.RT_NEAREST, 524288)])
+def test_both_sides_of_the_few_fragments_rule(sizes, S, filt, F):
+    """Where a lane per lookup gives way to a thread per fragment, by sample count and filter."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    uv, d, obj = _inputs(F, S, S, 3)
+    (a, ea), (b, eb) = _both(sizes, 5, uv, d, obj, filt)
+    np.testing.assert_array_equal(a.view(np.int32), b.view(np.int32))
+    assert ea == eb == api.RT_OK and a.any() and not a[obj < 0].any()
