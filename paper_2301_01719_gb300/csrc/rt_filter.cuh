@@ -177,10 +177,16 @@ __device__ __forceinline__ float filter_bits(const TexDesc& d, const Lookup<FILT
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const Idx o = r ? o1 : o0;
+            f32x2 q[4];
+#ifdef RADTEX_CHECKED
+            // every tap by itself: a checked index decides which bit is read
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[k] = pack2(texel(pl[k] + o), texel(pl[k] + o + u1));
+#else
             unsigned lo[4], hi[4], sh[4];  // the word of the first bucket's bit, the next one's, the bit
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const Idx a = (Idx)checked_texel(d, (int64_t)(pl[k] + o));
+                const Idx a = pl[k] + o;
                 if (KIND == kBitsWords) {
                     lo[k] = __ldg(words + ((pl[k] >> 5) + (o >> 5)));
                     sh[k] = (unsigned)o & 31u;
@@ -192,16 +198,13 @@ __device__ __forceinline__ float filter_bits(const TexDesc& d, const Lookup<FILT
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (u1 == 1u && sh[k] == 31u) {
-                    const Idx b = (Idx)checked_texel(d, (int64_t)(pl[k] + o + 1));
-                    hi[k] = __ldg(words + (b >> 5));
-                }
-            f32x2 q[4];
+                if (u1 == 1u && sh[k] == 31u) hi[k] = __ldg(words + ((pl[k] + o + 1) >> 5));
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const unsigned x = __funnelshift_r(lo[k], hi[k], sh[k]);  // the two bits, lowest first
                 q[k] = pack2(value(x), value(x >> u1));
             }
+#endif
             const float2 c = unpack2(lerp2(lerp2(q[0], q[1], ws), lerp2(q[2], q[3], ws), wt));
             row[r] = lerpf(c.x, c.y, L.u.w);
         }

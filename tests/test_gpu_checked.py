@@ -185,3 +185,42 @@ def test_accesses_past_the_limit_are_redirected_and_reported(ctx, path, filt):
     assert api.rt_get_error(ctx) == api.RT_OK
     assert np.max(np.abs(out.cpu().numpy() - ref_full)) <= COLOUR_TOL
     api.rt_destroy_texture(ctx, oid)
+
+
+@pytest.mark.parametrize("W,H", [(32, 32), (37, 23)])  # planes of whole words, and not
+@pytest.mark.parametrize("S,F", [(3, 3001), (4, 98304), (4, 3001)])  # a thread per fragment, and a lane per lookup
+@pytest.mark.parametrize("filt", [api.RT_ANGULAR_BILINEAR, api.RT_QUADRILINEAR])
+def test_bits_past_the_limit_are_redirected_and_reported(W, H, S, F, filt):
+    """rt_shade_multi on a context of bits: a bit past the limit (inside a word of bits that are not)
+    reads as texel 0."""
+    _checked_only()
+    n, T = 8, 3001
+    rng = np.random.default_rng(W + S)
+    bits = rng.integers(0, 2, (H * n, W * n), dtype=np.uint8)
+    uv = rng.random((F, 2), dtype=np.float32)
+    d = rng.standard_normal((F, S, 3))
+    d[..., 2] = np.abs(d[..., 2])
+    d = (d / np.linalg.norm(d, axis=2, keepdims=True)).astype(np.float32)
+    own = api.Context(0)
+    oid = api.rt_create_texture(own, W, H, n, api.RT_BIT1, api.RT_LAYOUT_ATLAS,
+                                to_dev(np.repeat(bits[..., None], 4, axis=2).astype(np.float32)))
+    obj = np.full(F, oid, np.int32)
+    limit = W * H * n * n // 2 + 13
+    assert api.rt_checked_limit_extent(own, oid, limit) == api.RT_OK
+    out = api.rt_shade_multi(own, to_dev(uv), to_dev(d), to_dev(obj), filt)[-T:].cpu().numpy()
+    assert api.rt_get_error(own) == api.RT_ERR_OUT_OF_BOUNDS
+    assert api.rt_get_error(own) == api.RT_OK
+
+    def reference(b):
+        ref, flags = oracle.shade([oracle.bit_texture(b, W, H, n)], np.repeat(uv[-T:], S, axis=0),
+                                  d[-T:].reshape(-1, 3), np.zeros(T * S, np.int32), filt)
+        assert flags == 0
+        return ref.reshape(T, S, 4).mean(axis=1)
+
+    planes = bits.reshape(H, n, W, n).transpose(1, 3, 0, 2).reshape(-1).copy()
+    planes[limit:] = planes[0]
+    redirected = planes.reshape(n, n, H, W).transpose(2, 0, 3, 1).reshape(H * n, W * n)
+    ref = reference(np.ascontiguousarray(redirected))
+    assert np.max(np.abs(out - ref)) <= COLOUR_TOL
+    assert np.sum(np.any(np.abs(reference(bits) - ref) > 1e-3, axis=1)) > 100
+    own.close()
