@@ -302,6 +302,9 @@ __device__ __forceinline__ float4 member_texel(const TexDesc& d, uint32_t at, in
         const int j = (int)(at / (uint32_t)d.W), i = (int)(at - (uint32_t)j * d.W);
         return load_texel<FMT>(d.base, texel_index<RT_LAYOUT_ATLAS>(d, i, j, p % d.n, p / d.n), 1.0f);
     }
+#ifdef RADTEX_CHECKED
+    at = (uint32_t)checked_slot(d, at, d.plane);
+#endif
     const float sc = FMT == RT_E4M3_BUCKET_SCALE ? __ldg(d.scale + at) : 1.0f;
     return load_texel<FMT>(d.base, checked_texel(d, (int64_t)p * d.plane + at), sc);
 }
