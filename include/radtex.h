@@ -223,7 +223,10 @@ rt_status rt_kmeans_assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const floa
  * earlier rt_kmeans_assign_tc of the same texture left in it (same object,
  * texels unchanged since, same K and scratch, ordered before this call), so the
  * bucket vectors are not converted again.  The Lloyd steps of one encoding call
- * it after the first assignment. */
+ * it after the first assignment.  A scratch of another object or K, of the
+ * object before it was created, filled or baked anew, or of no assignment raises
+ * RT_ERR_INVALID_ARG in rt_get_error, and the results are then undefined (a
+ * borrowed buffer's owner must not write it in between: that goes unseen). */
 rt_status rt_kmeans_reassign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* centroids, uint32_t* index,
                                 float* dist, void* scratch, int64_t scratch_bytes, rt_stream_t stream);
 

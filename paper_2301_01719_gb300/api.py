@@ -192,10 +192,20 @@ def rt_kmeans_assign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Tens
 def rt_kmeans_reassign_tc(ctx: Context, obj_id: int, K: int, centroids: torch.Tensor, index: torch.Tensor,
                           dist: torch.Tensor | None, scratch: TcScratch, stream=None) -> torch.Tensor:
     """rt_kmeans_assign_tc with other centroids, on the scratch that an earlier call of it on the
-    same (unchanged) texture left: the bucket vectors are not converted again."""
+    same (unchanged) texture with the same K left: the bucket vectors are not converted again
+    (another scratch: RT_ERR_INVALID_ARG in rt_get_error)."""
+    w, h, n, _, _ = _texture_info(ctx, obj_id)
     _check(centroids, "centroids", torch.float32, 4)
-    if centroids.numel() != K * rt_texture_info(ctx, obj_id)["n"] ** 2 * 4:
+    if centroids.numel() != K * n ** 2 * 4:
         raise ValueError("centroids must hold K x n x n x 4 values")
+    _check(index, "index", torch.uint32 if getattr(index, "dtype", None) is torch.uint32 else torch.int32)
+    if dist is not None:
+        _check(dist, "dist", torch.float32)
+    for t in (index,) if dist is None else (index, dist):
+        if t.numel() != w * h or t.device != centroids.device:
+            raise ValueError("index and dist must hold one entry per bucket on the centroids' device")
+    if scratch.buf.device != centroids.device:
+        raise ValueError("scratch must live on the centroids' device")
     _lib.call("rt_kmeans_reassign_tc", ctx.handle, int(obj_id), int(K), _ptr(centroids), _ptr(index), _ptr(dist),
               scratch.ptr, int(scratch.nbytes), _stream(stream, centroids.device))
     return index

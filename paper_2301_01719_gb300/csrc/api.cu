@@ -2,6 +2,7 @@
 // texture table, argument validation, kernel launches and the status model.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -28,6 +29,7 @@ struct rt_ctx {
     int tile[2][3][4];                   // per pass (forward, backward) and filter: tw, th, bx, by of the batched kernels
     long long* det[RT_MAX_OBJECTS];      // fixed-point gradient sums of the deterministic mode
     uint32_t* index[RT_MAX_OBJECTS];     // palette index maps the library copied
+    uint64_t texels[RT_MAX_OBJECTS];     // a number of the object's present texels (new_texels)
     int spec = -1;                       // the format (+ kSpecPalette) shared by all objects in clamp mode, else -1
     int bits = rt::kBitsNone;            // how the bits are indexed if all objects are bit textures in clamp mode
     uint32_t wait_limit = 0;             // polls of a bounded device wait before it gives up (0: the default)
@@ -127,6 +129,13 @@ int table_bits(const rt_ctx* ctx) {
     return bits;
 }
 
+// Every creation, fill and bake of a texture gives its texels a number no others
+// have had in this process (writes into a borrowed buffer go unseen).
+void new_texels(rt_ctx* ctx, int o) {
+    static std::atomic<uint64_t> last{0};
+    ctx->texels[o] = last.fetch_add(1, std::memory_order_relaxed) + 1;
+}
+
 rt_status upload_table(rt_ctx* ctx) {
     ctx->spec = table_spec(ctx);
     ctx->bits = table_bits(ctx);
@@ -185,6 +194,7 @@ rt_status rt_context_create(int cuda_device, rt_ctx** out) {
     std::memset(ctx->bytes, 0, sizeof(ctx->bytes));
     std::memset(ctx->det, 0, sizeof(ctx->det));
     std::memset(ctx->index, 0, sizeof(ctx->index));
+    std::memset(ctx->texels, 0, sizeof(ctx->texels));
     for (int p = 0; p < 2; ++p)
         for (int f = 0; f < 3; ++f) {
             ctx->tile[p][f][0] = 8;
@@ -350,6 +360,7 @@ static rt_status create_object(rt_ctx* ctx, int32_t w, int32_t h, int32_t n, int
     ctx->index[o] = index_ptr;
     if (index_ptr) ctx->bytes[o] += (int64_t)sizeof(uint32_t) * w * h;
     ctx->table[o] = d;
+    new_texels(ctx, o);
     if (o + 1 > ctx->n_obj) ctx->n_obj = o + 1;
     rt_status st = upload_table(ctx);
     if (st != RT_OK) {
@@ -441,6 +452,7 @@ rt_status rt_fill_bucket_lobes(rt_ctx* ctx, int32_t obj_id, const float* params,
     if (!ctx->owned[obj_id] || d.layout == rt::kLayoutPalette || d.fmt == RT_BIT1) return RT_ERR_UNSUPPORTED;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
+    new_texels(ctx, obj_id);
     return cuda_status(rt::launch_fill_lobes(params, ctx->owned[obj_id], ctx->scales[obj_id], d.layout, d.W, d.H, d.n,
                                              d.fmt,
                                              (cudaStream_t)stream));
@@ -462,6 +474,7 @@ rt_status rt_bake(rt_ctx* ctx, int32_t obj_id, rt_surface surface, const rt_bake
     if (d.layout == rt::kLayoutPalette || d.fmt == RT_BIT1) return RT_ERR_UNSUPPORTED;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
+    new_texels(ctx, obj_id);
     return cuda_status(rt::launch_bake(*scene, (int)surface, const_cast<void*>(d.base), ctx->scales[obj_id], d.W, d.H,
                                        d.n, d.fmt, d.layout, nullptr, 0, (cudaStream_t)stream));
 }
@@ -476,6 +489,7 @@ rt_status rt_bake_deferred(rt_ctx* ctx, int32_t obj_id, rt_surface surface, cons
     if (d.layout == rt::kLayoutPalette || d.fmt == RT_BIT1) return RT_ERR_UNSUPPORTED;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
+    new_texels(ctx, obj_id);
     return cuda_status(rt::launch_bake(*scene, (int)surface, const_cast<void*>(d.base), ctx->scales[obj_id], d.W, d.H,
                                        d.n, d.fmt, d.layout, ao_dirs, K, (cudaStream_t)stream));
 }
@@ -518,8 +532,8 @@ static rt_status assign_tc(rt_ctx* ctx, int32_t obj_id, int32_t K, const float* 
     if (scratch_bytes < rt::kmeans_tc_scratch_bytes(d.W, d.H, d.n, K)) return RT_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return RT_ERR_CUDA;
-    cudaError_t e = rt::launch_kmeans_assign_tc(d, K, centroids, index, dist, scratch, converted, ctx->d_status,
-                                                ctx->wait_limit, (cudaStream_t)stream);
+    cudaError_t e = rt::launch_kmeans_assign_tc(d, K, centroids, index, dist, scratch, ctx->texels[obj_id], converted,
+                                                ctx->d_status, ctx->wait_limit, (cudaStream_t)stream);
     return e == cudaErrorNotSupported ? RT_ERR_UNSUPPORTED : cuda_status(e);
 }
 

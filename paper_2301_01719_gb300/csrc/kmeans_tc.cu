@@ -405,9 +405,19 @@ __global__ void row_norms_kernel(const __half* __restrict__ X, int rows, int Dp,
 }
 
 // C: centroids (n, n, K, 4) FP32 -> FP16 rows (k, (t n + s) 4 + c), zero padding.
+// `tag` says what the scratch's X was converted from (the texels' generation and
+// K, which places the norms): written by an assignment that converts, compared by
+// one that does not (`converted`).
 __global__ void convert_c_kernel(const float4* __restrict__ C, int K, int planes, int Kp, int Dp,
-                                 __half* __restrict__ out) {
+                                 __half* __restrict__ out, ulonglong2* __restrict__ tag, ulonglong2 want,
+                                 bool converted, unsigned* status) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // (k, p) over Kp x Dp / 4
+    if (e == 0) {
+        if (!converted)
+            *tag = want;
+        else if (tag->x != want.x || tag->y != want.y)
+            atomicOr(status, ST_BAD_ARG);
+    }
     const int P4 = Dp / 4;
     if (e >= (int64_t)Kp * P4) return;
     const int k = (int)(e / P4), p = (int)(e - (int64_t)k * P4);
@@ -420,7 +430,7 @@ __global__ void convert_c_kernel(const float4* __restrict__ C, int K, int planes
 
 struct Layout {
     int64_t Bp, Dp, Kp;
-    size_t x_off, c_off, cn_off, xn_off, bytes;
+    size_t x_off, c_off, cn_off, xn_off, tag_off, bytes;
 };
 
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -434,7 +444,8 @@ inline Layout layout(int W, int H, int n, int K) {
     L.c_off = (size_t)round_up(L.Bp * L.Dp * 2, 1024);
     L.cn_off = L.c_off + (size_t)round_up(L.Kp * L.Dp * 2, 1024);
     L.xn_off = L.cn_off + (size_t)round_up(L.Kp * 4, 1024);
-    L.bytes = L.xn_off + (size_t)round_up(L.Bp * 4, 1024);
+    L.tag_off = L.xn_off + (size_t)round_up(L.Bp * 4, 1024);
+    L.bytes = L.tag_off + 1024;
     return L;
 }
 
@@ -517,8 +528,8 @@ static cudaError_t convert_x_fmt(const TexDesc& d, const Layout& L, __half* X, f
 int64_t kmeans_tc_scratch_bytes(int W, int H, int n, int K) { return (int64_t)tc::layout(W, H, n, K).bytes; }
 
 cudaError_t launch_kmeans_assign_tc(const TexDesc& d, int K, const float* C, uint32_t* index, float* dist,
-                                    void* scratch, bool converted, unsigned* status, uint32_t spin_limit,
-                                    cudaStream_t stream) {
+                                    void* scratch, uint64_t texels, bool converted, unsigned* status,
+                                    uint32_t spin_limit, cudaStream_t stream) {
     using namespace tc;
     const Layout L = layout(d.W, d.H, d.n, K);
     uint8_t* base = static_cast<uint8_t*>(scratch);
@@ -526,6 +537,7 @@ cudaError_t launch_kmeans_assign_tc(const TexDesc& d, int K, const float* C, uin
     __half* Ch = reinterpret_cast<__half*>(base + L.c_off);
     float* cn = reinterpret_cast<float*>(base + L.cn_off);
     float* xn = reinterpret_cast<float*>(base + L.xn_off);
+    ulonglong2* tag = reinterpret_cast<ulonglong2*>(base + L.tag_off);
     cudaError_t e;
     if (converted)
         e = cudaSuccess;
@@ -538,7 +550,9 @@ cudaError_t launch_kmeans_assign_tc(const TexDesc& d, int K, const float* C, uin
     if (e != cudaSuccess) return e;
     const int64_t ce = L.Kp * (L.Dp / 4);
     convert_c_kernel<<<(unsigned)((ce + 255) / 256), 256, 0, stream>>>(reinterpret_cast<const float4*>(C), K,
-                                                                        d.n * d.n, (int)L.Kp, (int)L.Dp, Ch);
+                                                                        d.n * d.n, (int)L.Kp, (int)L.Dp, Ch, tag,
+                                                                        make_ulonglong2(texels, (uint64_t)K),
+                                                                        converted, status);
     row_norms_kernel<<<(unsigned)((L.Kp * 32 + 255) / 256), 256, 0, stream>>>(Ch, (int)L.Kp, (int)L.Dp, cn,
                                                                               INFINITY, K);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

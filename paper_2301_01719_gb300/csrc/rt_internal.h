@@ -102,10 +102,11 @@ cudaError_t launch_world_backward(const TexDesc* table, int n_obj, const float* 
                                   float* dL_duv, float* dL_ddir, float* dL_dnrm, bool accumulate, bool deterministic,
                                   unsigned* status, cudaStream_t stream);
 int64_t kmeans_tc_scratch_bytes(int W, int H, int n, int K);
-// converted: the scratch holds the bucket vectors and their norms already.
+// texels: a number of the texture's present texels.  converted: the scratch holds their bucket vectors
+// and norms already (else ST_BAD_ARG).
 cudaError_t launch_kmeans_assign_tc(const TexDesc& d, int K, const float* C, uint32_t* index, float* dist,
-                                    void* scratch, bool converted, unsigned* status, uint32_t spin_limit,
-                                    cudaStream_t stream);
+                                    void* scratch, uint64_t texels, bool converted, unsigned* status,
+                                    uint32_t spin_limit, cudaStream_t stream);
 cudaError_t launch_kmeans_init(const TexDesc& d, int K, const int32_t* buckets, float* C, unsigned* status,
                                cudaStream_t stream);
 cudaError_t launch_kmeans_assign(const TexDesc& d, int K, const float* C, uint32_t* index, float* dist,

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import synth
 from paper_2301_01719_gb300 import api
 
 pytestmark = pytest.mark.gpu
@@ -134,3 +135,58 @@ def test_tensor_core_distances_of_few_buckets_with_many_planes(ctx, w, h, n, K, 
     assert api.rt_get_error(ctx) == api.RT_OK
     api.rt_destroy_texture(ctx, oid)
     del keep
+
+
+def _reassign_setup(ctx, w=24, h=10, n=4, K=6):
+    oid, _, _ = _texture(ctx, np.random.default_rng(1).random((n, n, h, w, 4), dtype=np.float32), api.RT_F16)
+    C = torch.rand((n, n, K, 4), device="cuda")
+    scratch = api.TcScratch(api.rt_kmeans_tc_scratch_bytes(w, h, n, K + 300), C.device)  # for another K too
+    index = torch.empty((h, w), dtype=torch.int32, device="cuda")
+    return oid, C, scratch, index
+
+
+@pytest.mark.parametrize("change", ["none", "never converted", "other object", "other K", "baked", "filled",
+                                    "created anew"])
+def test_reassignment_reports_a_scratch_of_other_texels(ctx, change):
+    """The scratch carries what it was converted from; a reassignment on another one is an error."""
+    w, h, n, K = 24, 10, 4, 6
+    oid, C, scratch, index = _reassign_setup(ctx)
+    ids = [oid]
+    scratch.buf.zero_()
+    if change != "never converted":
+        api.rt_kmeans_assign_tc(ctx, oid, K, C, index, scratch=scratch)
+    if change == "other object":
+        ids.append(api.rt_create_texture(ctx, w, h, n, api.RT_F16))
+    elif change == "other K":
+        K = 300
+        C = torch.rand((n, n, K, 4), device="cuda")
+    elif change == "baked":
+        api.rt_bake(ctx, oid, api.RT_SURFACE_SPHERE, synth.bake_scene(3))
+    elif change == "filled":
+        api.rt_fill_bucket_lobes(ctx, oid, torch.rand((h, w, 8), device="cuda"))
+    elif change == "created anew":
+        api.rt_destroy_texture(ctx, oid)
+        assert api.rt_create_texture(ctx, w, h, n, api.RT_F16) == oid
+    assert api.rt_get_error(ctx) == api.RT_OK
+    api.rt_kmeans_reassign_tc(ctx, ids[-1], K, C, index, None, scratch)
+    assert api.rt_get_error(ctx) == (api.RT_OK if change == "none" else api.RT_ERR_INVALID_ARG)
+    api.rt_kmeans_assign_tc(ctx, ids[-1], K, C, index, scratch=scratch)  # converts: the scratch is good again
+    api.rt_kmeans_reassign_tc(ctx, ids[-1], K, C, index, None, scratch)
+    assert api.rt_get_error(ctx) == api.RT_OK
+    for o in ids:
+        api.rt_destroy_texture(ctx, o)
+
+
+def test_reassignment_checks_its_tensors(ctx):
+    oid, C, scratch, index = _reassign_setup(ctx)
+    api.rt_kmeans_assign_tc(ctx, oid, 6, C, index, scratch=scratch)
+    dist = torch.empty((10, 24), device="cuda")
+    for bad_index, bad_dist, error in ((None, None, TypeError), (index.cpu(), None, TypeError),
+                                       (index.long(), None, TypeError), (index[:, ::2], None, ValueError),
+                                       (index[:5].clone(), None, ValueError), (index, dist.double(), TypeError),
+                                       (index, dist[:9].clone(), ValueError), (index, dist.cpu(), TypeError)):
+        with pytest.raises(error):
+            api.rt_kmeans_reassign_tc(ctx, oid, 6, C, bad_index, bad_dist, scratch)
+    api.rt_kmeans_reassign_tc(ctx, oid, 6, C, index.view(torch.uint32), dist, scratch)
+    assert api.rt_get_error(ctx) == api.RT_OK
+    api.rt_destroy_texture(ctx, oid)
