@@ -378,14 +378,15 @@ __global__ void __launch_bounds__(CTHREADS) convert_x_kernel(TexDesc d, int Dp, 
         }
         __syncthreads();
     }
-    if (SPLIT) return;
+    if constexpr (!SPLIT) {
 #pragma unroll
-    for (int r = 0; r < CB / (CTHREADS / 32); ++r) {
-        float s = norm[r];
-        for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        const int bl = warp * (CB / (CTHREADS / 32)) + r;
-        const int bi = i0 + (bl & (CI - 1)), bj = j0 + bl / CI;
-        if (lane == 0 && bi < d.W && bj < d.H) xn[(int64_t)bj * d.W + bi] = s;
+        for (int r = 0; r < CB / (CTHREADS / 32); ++r) {
+            float s = norm[r];
+            for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            const int bl = warp * (CB / (CTHREADS / 32)) + r;
+            const int bi = i0 + (bl & (CI - 1)), bj = j0 + bl / CI;
+            if (lane == 0 && bi < d.W && bj < d.H) xn[(int64_t)bj * d.W + bi] = s;
+        }
     }
 }
 
