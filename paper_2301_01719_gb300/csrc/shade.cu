@@ -72,9 +72,13 @@ __global__ void __launch_bounds__(kShadeThreads) locate_kernel(const TexDesc* __
 // World-space forward and lookup (Eq. 1a with a per-fragment normal): the
 // streamer of the tangent-space kernels with a fourth staged stream, the
 // normal, over the flat fragment stream or, TILED, over screen tiles of a batch
-// of frames.
+// of frames.  Held to 64 registers and 8 blocks per SM, but for the dispatching
+// quadrilinear kernels, which would spill (110 registers, 4 blocks): left to itself
+// the compiler took 66 and 71 for the dispatching nearest and angular-bilinear ones,
+// 7 blocks, and 4 frames of 1080p on FP16 took 84 and 92 us in the flat call instead of
+// 73 and 80 (9 or 10 blocks: no better).
 template <int FILTER, bool TILED, int SPEC>
-__global__ void __launch_bounds__(kShadeThreads, SPEC >= 0 ? 8 : 1) world_shade_kernel(const TexDesc* __restrict__ table, int n_obj,
+__global__ void __launch_bounds__(kShadeThreads, SPEC >= 0 || FILTER != RT_QUADRILINEAR ? 8 : 1) world_shade_kernel(const TexDesc* __restrict__ table, int n_obj,
                                                                     const float* __restrict__ uv,
                                                                     const float* __restrict__ dir,
                                                                     const float* __restrict__ nrm,
