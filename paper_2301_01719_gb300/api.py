@@ -34,9 +34,15 @@ def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
 
 
+# torch.cuda.current_stream(device).cuda_stream without the Stream object (2 us), in the torch releases that have it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream, device) -> int:
-    if stream is None:  # torch.cuda.current_stream(device).cuda_stream without the Stream object (2 us)
-        return torch._C._cuda_getCurrentRawStream(device.index)
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(device.index)
+        stream = torch.cuda.current_stream(device)
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
