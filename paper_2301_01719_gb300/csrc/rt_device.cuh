@@ -89,10 +89,6 @@ __device__ __forceinline__ int checked_slot(const TexDesc& d, int64_t slot, int6
 }
 #endif
 
-__device__ __forceinline__ bool finite3(float a, float b, float c) {
-    return isfinite(a) && isfinite(b) && isfinite(c);
-}
-
 // Eq. 3 applied to A = sqrt(2) h_xy / |h|, the equisolid projection of a
 // half-way vector h: h = (I_x, I_y, I_z + 1) in the tangent frame (Eq. 1b) or
 // h = I + N in any frame (Eq. 1a).  Since A is a positive multiple of h_xy,
@@ -360,17 +356,6 @@ __device__ __forceinline__ float4 load_texel<RT_E4M3_BUCKET_SCALE>(const void* b
     float2 b = e4m3x2_to_float2((unsigned short)(r >> 16));
     return make_float4(a.x * scale, a.y * scale, b.x * scale, b.y * scale);
 }
-
-__device__ __forceinline__ float4 lerp4(float4 a, float4 b, float w) {
-    return make_float4(fmaf(w, b.x - a.x, a.x), fmaf(w, b.y - a.y, a.y), fmaf(w, b.z - a.z, a.z),
-                       fmaf(w, b.w - a.w, a.w));
-}
-
-__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
-    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-}
-
-__device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
 // RGBA held as two packed FP32 pairs, filtered with the paired FP32 FMA of
 // sm_100+ (fma.rn.f32x2 / sub.rn.f32x2): the same roundings as the scalar

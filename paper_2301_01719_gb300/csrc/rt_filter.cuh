@@ -16,20 +16,6 @@ namespace rt {
 
 // The four texels (s0,t0) (s1,t0) (s0,t1) (s1,t1) of bucket (i, j).
 template <int FMT, int LAYOUT>
-__device__ __forceinline__ void load_quad(const TexDesc& d, int i, int j, const Axis& s, const Axis& t, float4& t00,
-                                          float4& t10, float4& t01, float4& t11) {
-    float sc = 1.0f;
-    if (FMT == RT_E4M3_BUCKET_SCALE) sc = __ldg(d.scale + bucket_slot<LAYOUT>(d, i, j));
-    t00 = load_texel<FMT>(d.base, texel_index<LAYOUT>(d, i, j, s.k0, t.k0), sc);
-    t10 = load_texel<FMT>(d.base, texel_index<LAYOUT>(d, i, j, s.k1, t.k0), sc);
-    t01 = load_texel<FMT>(d.base, texel_index<LAYOUT>(d, i, j, s.k0, t.k1), sc);
-    t11 = load_texel<FMT>(d.base, texel_index<LAYOUT>(d, i, j, s.k1, t.k1), sc);
-}
-
-// Addresses of the taps.  PLANES / QUADS: the four in-bucket texels (s0|s1,
-// t0|t1) select four planes (64-bit base indices), the (up to) four buckets
-// select spatial offsets inside a plane (32-bit, w h < 2^31).
-template <int FMT, int LAYOUT>
 __device__ __forceinline__ void load_quadP(const TexDesc& d, int i, int j, const Axis& s, const Axis& t, P4& t00,
                                            P4& t10, P4& t01, P4& t11) {
     float sc = 1.0f;
@@ -40,6 +26,9 @@ __device__ __forceinline__ void load_quadP(const TexDesc& d, int i, int j, const
     t11 = load_texelP<FMT>(d.base, texel_index<LAYOUT>(d, i, j, s.k1, t.k1), sc);
 }
 
+// Addresses of the taps.  PLANES / QUADS: the four in-bucket texels (s0|s1,
+// t0|t1) select four planes (64-bit base indices), the (up to) four buckets
+// select spatial offsets inside a plane (32-bit, w h < 2^31).
 // The planes (64-bit bases, k = (s0,t0) (s1,t0) (s0,t1) (s1,t1)) and the spatial
 // offsets (b = (u0,v0) (u1,v0) (u0,v1) (u1,v1)) of a quadrilinear lookup's 16 taps
 // on a PLANES / QUADS / palette texture: tap (b, k) is texel pl[k] + o[b].
