@@ -115,8 +115,22 @@ cudaError_t launch_backward(const TexDesc* table, int n_obj, const float* uv, co
 // the tangent-space backward with the normal as a fourth staged stream, over
 // the flat fragment stream or, TILED, over screen tiles of a batch of frames.
 // dL/dI = dL/dN, since A depends on h = I + N only.
+// The dispatching kernels' blocks per SM: left to itself the compiler takes 136
+// (tiled) and 128 registers for the quadrilinear ones, 85 for the angular-bilinear
+// ones.  4 frames of 1080p, FP16 and FP32 objects, coordinate gradients / texel
+// gradients as well, us (136, 128, 85 -> here): quadrilinear in tiles 223 -> 189 / 572 -> 542
+// (5 blocks: 188 / 551), flat 217 -> 173 / 562 -> 517 (4 blocks: 182 / 518); angular-bilinear in
+// tiles 146 -> 127, flat 144 -> 125 (6 blocks: 133, 134).  The deterministic ones: 4 blocks,
+// quadrilinear in tiles 1869 -> 1844.
 template <int FILTER, bool DET, bool TILED, int SPEC>
-__global__ void __launch_bounds__(kBackThreads, SPEC >= 0 ? 6 : 1) world_backward_kernel(
+constexpr int world_backward_blocks() {
+    if (SPEC >= 0) return 6;
+    if (DET) return 4;
+    return FILTER == RT_QUADRILINEAR ? (TILED ? 4 : 5) : FILTER == RT_ANGULAR_BILINEAR ? 7 : 1;
+}
+
+template <int FILTER, bool DET, bool TILED, int SPEC>
+__global__ void __launch_bounds__(kBackThreads, world_backward_blocks<FILTER, DET, TILED, SPEC>()) world_backward_kernel(
     const TexDesc* __restrict__ table, int n_obj, const float* __restrict__ uv, const float* __restrict__ dir,
     const float* __restrict__ nrm, const int32_t* __restrict__ obj, int64_t F, Tiling tiling,
     const float* __restrict__ dL_dout,
@@ -180,8 +194,11 @@ static cudaError_t launch_world_backward_t(const TexDesc* table, int n_obj, cons
                                            const float* dL_dout, const GradTable& grads, bool any_grad, float* dL_duv,
                                            float* dL_ddir, float* dL_dnrm, bool accumulate, unsigned* status,
                                            cudaStream_t stream) {
-    const unsigned grid = persistent_grid<world_backward_kernel<FILTER, DET, TILED, SPEC>>(kBackThreads,
-                                          chunk_count_host(T, F, kBackWarps));
+    // with texel gradients more warps only queue at the reductions: angular-bilinear, 7 blocks 426 us in
+    // tiles and 417 flat, 6 415 and 401, 5 413 and 393, 4 419 and 404
+    const int most = FILTER == RT_ANGULAR_BILINEAR && SPEC < 0 && any_grad ? 5 : 0;
+    const unsigned grid = persistent_grid<world_backward_kernel<FILTER, DET, TILED, SPEC>>(
+        kBackThreads, chunk_count_host(T, F, kBackWarps), most);
     world_backward_kernel<FILTER, DET, TILED, SPEC><<<grid, kBackThreads, 0, stream>>>(
         table, n_obj, uv, dir, nrm, obj, F, T, dL_dout, grads, any_grad, dL_duv, dL_ddir, dL_dnrm, accumulate,
         status);
