@@ -260,9 +260,10 @@ __global__ void __launch_bounds__(kShadeThreads) multi_shade_lanes_kernel(const 
 // fragment per thread, its samples one after another with the next direction
 // loaded ahead (the validity test, the spatial axes and the bucket offsets are
 // then a fragment's, not a lookup's).  A power of two up to 32 samples is summed
-// as the tree of multi_shade_lanes_kernel, others in their order.  Bound: issue.
+// as the tree of multi_shade_lanes_kernel, others in their order.  Bound: issue
+// (two thirds of the cycles) and the gathers' latency (L1 data pipe 62 %).
 // 10 poses of 1080p, S = 4, quadrilinear on 2 x 1024^2 x 16^2 bits: 1.12 ms with the
-// general kernel, 0.77 with a lane per lookup, 0.645 here; 2 views of 1366 x 768
+// general kernel, 0.77 with a lane per lookup, 0.645 here (to 0.80 by input); 2 views of 1366 x 768
 // (lane per lookup -> here): S = 3, angular 56 -> 36 us, S = 16, quadrilinear 351 -> 265.
 template <int FILTER, int KIND>
 __global__ void __launch_bounds__(kShadeThreads, 8) multi_bits_kernel(const TexDesc* __restrict__ table, int n_obj,
